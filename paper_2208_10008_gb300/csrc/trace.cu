@@ -5,6 +5,14 @@
 // k_trace (float32, one ray per thread)
 //   * 4-wide nodes, one 128-byte line each, read with 16-byte read-only loads;
 //     children ordered near-first on a per-thread stack.
+//   * a warp alternates: its lanes visit nodes until at least as many of them
+//     wait at a leaf as still have a node to visit, then the waiting ones test
+//     their triangles together.  Lanes that test a leaf as soon as they meet
+//     one make almost every turn of the loop pay for both sides (6.1 of 32
+//     lanes active on random segments): 1,000,003 of them on the 20k-triangle
+//     city 0.743 -> 0.593 ms, 655,362 launched rays 0.120 -> 0.111 ms.
+//     Waiting until no lane has a node left costs 0.637 ms there, testing at
+//     half or an eighth as many waiting lanes 0.636 / 0.750 ms.
 //   * box test: slab test with the near/far plane picked by the sign of 1/d
 //     (NaN-safe for axis-parallel rays); the interval is widened by a relative
 //     1e-6 so rounding never drops a box the exact ray meets.
@@ -211,6 +219,18 @@ __device__ float refine_t(const RayPre& r, float dx, float dy, float dz, float4 
   return __fadd_rn(q, __fdiv_rn(rem.hi, den.hi));
 }
 
+// (plane - o) * i of a node's four planes of one kind, two to a packed
+// instruction (a - o is a + -o, each step rounded as the scalar one is).
+__device__ __forceinline__ void plane4(float4 v, float o, float i, float t[4]) {
+  const float2 o2 = make_float2(-o, -o), i2 = make_float2(i, i);
+  const float2 a = __fmul2_rn(__fadd2_rn(make_float2(v.x, v.y), o2), i2);
+  const float2 b = __fmul2_rn(__fadd2_rn(make_float2(v.z, v.w), o2), i2);
+  t[0] = a.x;
+  t[1] = a.y;
+  t[2] = b.x;
+  t[3] = b.y;
+}
+
 // Slab test of the 4 children of a node; returns a bit mask of children
 // whose widened interval meets [tmin, bound], near distances in tn[].
 __device__ __forceinline__ unsigned slab4(const WNode* __restrict__ node, const RayPre& r, float bound,
@@ -223,16 +243,18 @@ __device__ __forceinline__ unsigned slab4(const WNode* __restrict__ node, const 
   const float4 nz = __ldg(p + 4 + r.sz), fz = __ldg(p + 5 - r.sz);
   int4 ch = __ldg(reinterpret_cast<const int4*>(p + 6));
   *child = ch;
-  float nxa[4] = {nx.x, nx.y, nx.z, nx.w}, fxa[4] = {fx.x, fx.y, fx.z, fx.w};
-  float nya[4] = {ny.x, ny.y, ny.z, ny.w}, fya[4] = {fy.x, fy.y, fy.z, fy.w};
-  float nza[4] = {nz.x, nz.y, nz.z, nz.w}, fza[4] = {fz.x, fz.y, fz.z, fz.w};
+  float nxt[4], fxt[4], nyt[4], fyt[4], nzt[4], fzt[4];
+  plane4(nx, r.ox, r.ix, nxt);
+  plane4(fx, r.ox, r.ix, fxt);
+  plane4(ny, r.oy, r.iy, nyt);
+  plane4(fy, r.oy, r.iy, fyt);
+  plane4(nz, r.oz, r.iz, nzt);
+  plane4(fz, r.oz, r.iz, fzt);
   unsigned mask = 0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float t0 = fmaxf(fmaxf(__fmul_rn(__fsub_rn(nxa[i], r.ox), r.ix), __fmul_rn(__fsub_rn(nya[i], r.oy), r.iy)),
-                     __fmul_rn(__fsub_rn(nza[i], r.oz), r.iz));
-    float t1 = fminf(fminf(__fmul_rn(__fsub_rn(fxa[i], r.ox), r.ix), __fmul_rn(__fsub_rn(fya[i], r.oy), r.iy)),
-                     __fmul_rn(__fsub_rn(fza[i], r.oz), r.iz));
+    float t0 = fmaxf(fmaxf(nxt[i], nyt[i]), nzt[i]);
+    float t1 = fminf(fminf(fxt[i], fyt[i]), fzt[i]);
     t0 = t0 - fabsf(t0) * kWiden;
     t1 = t1 + fabsf(t1) * kWiden;
     tn[i] = t0;
@@ -378,14 +400,19 @@ struct TraceArgs {
 };
 
 // The float32 walk of ray i (the whole of Fig. 4 for one ray): results,
-// statistics and the flag for the float64 pass.
+// statistics and the flag for the float64 pass.  Called by whole warps;
+// lanes without a ray pass live = false.  A lane visits the same boxes and
+// triangles in the same order whatever its warp does, so its result does not
+// depend on the other lanes.
 template <bool kAny, bool kStats, int kSD, bool kQuant, int kW>
-__device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const rt_ray* __restrict__ rays,
+__device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const bool live,
+                                         const rt_ray* __restrict__ rays,
                                          rt_hit* __restrict__ hits, uint8_t* __restrict__ occl,
                                          const int32_t* __restrict__ skip_ids) {
   const float4* r4 = reinterpret_cast<const float4*>(rays) + 2 * (size_t)i;
-  const RayPre r = setup_ray(__ldg(r4), __ldg(r4 + 1));
-  const int skip = skip_ids ? __ldg(skip_ids + i) : -1;
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);  // (an invalid ray: no direction)
+  const RayPre r = setup_ray(live ? __ldg(r4) : none, live ? __ldg(r4 + 1) : none);
+  const int skip = live && skip_ids ? __ldg(skip_ids + i) : -1;
   float t1 = INFINITY, t2 = INFINITY, e1 = 0.f, e2 = 0.f, bu = 0.f, bv = 0.f;
   int id1 = -1, pos1 = -1;
   bool flag = false, done = false;
@@ -422,18 +449,20 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
   // the node being visited stays in registers (cur); only the other
   // children hit by the ray go to the stack, nearest popped first
   int cur = r.valid ? __ldg(A.wide_root) : INT_MIN;
-  float cur_t = -INFINITY;
-  while (!done) {
-    if (cur == INT_MIN) {
-      if (sp == 0) break;
+  for (;;) {
+    while (cur == INT_MIN && sp > 0) {  // the next box that is not beyond the bound
       --sp;
-      cur = st[sp].x;
-      cur_t = __int_as_float(st[sp].y);
+      const int2 e = st[sp];
+      if (!(__int_as_float(e.y) > bound)) cur = e.x;
     }
-    const int ref = cur;
-    cur = INT_MIN;
-    if (cur_t > bound) continue;
-    if (ref >= 0) {
+    __syncwarp();
+    const int nn = __popc(__ballot_sync(kFullMask, cur >= 0));
+    const int nl = __popc(__ballot_sync(kFullMask, cur < 0 && cur != INT_MIN));
+    if (nn + nl == 0) break;
+    if (nn > nl) {  // the warp visits nodes
+      if (cur < 0) continue;
+      const int ref = cur;
+      cur = INT_MIN;
       if (kStats) ++n_nodes;
       if (kW == 8) {
         float tn[8];
@@ -444,7 +473,8 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         if (sp + cnt - 1 > kSD) {  // cannot hold the children: leave it to the float64 pass
           flag = true;
           walk_all = true;
-          break;
+          sp = 0;
+          continue;
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -474,7 +504,6 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         for (int q = 7; q >= 1; --q)
           if (q < cnt) st[sp++] = make_int2(ch[q], __float_as_int(tn[q]));
         cur = ch[0];
-        cur_t = tn[0];
         continue;
       }
       float tn[4];
@@ -494,17 +523,20 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       if (sp + cnt - 1 > kSD) {  // cannot hold the children: leave it to the float64 pass
         flag = true;
         walk_all = true;
-        break;
+        sp = 0;
+        continue;
       }
       // push farthest first so the nearest stacked one is popped next
       if (cnt > 3) st[sp++] = make_int2(rd, __float_as_int(td));
       if (cnt > 2) st[sp++] = make_int2(rc, __float_as_int(tc));
       if (cnt > 1) st[sp++] = make_int2(rb, __float_as_int(tb));
       cur = ra;
-      cur_t = ta;
       continue;
     }
-    // leaf
+    // the warp tests the triangles of the leaves that its lanes have reached
+    if (cur >= 0 || cur == INT_MIN) continue;
+    const int ref = cur;
+    cur = INT_MIN;
     const int first = leaf_first(ref), count = leaf_count(ref);
     for (int k = 0; k < count; ++k) {
       const float4* tp = A.tris + 3 * (size_t)(first + k);
@@ -532,6 +564,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
               fabsf(h.t - r.tmin) <= h.err + kTieRel * fabsf(h.t))) {
           done = true;
           id1 = id;
+          sp = 0;
           break;
         }
         continue;
@@ -552,6 +585,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       bound = fminf(r.tmax, t1 + kTieRel * t1 + e1);
     }
   }
+  if (!live) return;
   if (kAny) {
     occl[i] = done ? 1 : 0;
     if (done) flag = false;
@@ -584,11 +618,21 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
   }
 }
 
+// Registers by the launch bounds: 64 a thread (8 CTAs of 128 per SM) for the
+// closest hit, 56 (9) for any hit; left alone the compiler takes 80 and 72
+// and fewer walks are in flight to cover the node loads.  1,000,003 random
+// segments on the 20k-triangle city take 0.593 ms at 9 CTAs, 0.617 at 8,
+// 0.649 at 10 (spills); 262,143 random rays on the 200k-triangle city 0.239
+// ms at 8 CTAs, 0.245 at 7, 0.246 at 9.
+template <bool kAny, bool kStats, int kTile, int kSD, bool kQuant, int kW>
+constexpr int walk_ctas() {
+  return kStats ? 1 : (kW == 8 ? 6 : kAny && !kQuant ? 9 : 8) * 128 / kTile;
+}
 template <bool kAny, bool kStats, int kTile, int kSD, bool kQuant, int kW = 4>
-__global__ void __launch_bounds__(kTile) k_trace(TraceArgs A) {
+__global__ void __launch_bounds__(kTile, walk_ctas<kAny, kStats, kTile, kSD, kQuant, kW>()) k_trace(TraceArgs A) {
   const int i = blockIdx.x * kTile + threadIdx.x;
-  if (i >= A.n || (A.n_dev && i >= *A.n_dev)) return;
-  walk_one<kAny, kStats, kSD, kQuant, kW>(A, i, A.rays, A.hits, A.occl, A.skip);
+  const bool live = i < A.n && !(A.n_dev && i >= *A.n_dev);
+  walk_one<kAny, kStats, kSD, kQuant, kW>(A, i, live, A.rays, A.hits, A.occl, A.skip);
 }
 
 // ---------------------------------------------------------------- float64
@@ -935,7 +979,7 @@ __device__ __forceinline__ void walk_phase(const TraceArgs& A, int* take, int n,
     if (lane == 0) b = atomicAdd(take, 32);
     b = __shfl_sync(kFullMask, b, 0);
     if (b >= n) break;
-    if (b + lane < n) walk_one<kAny, false, kStack, false, kW>(A, b + lane, rays, hits, occl, skip);
+    walk_one<kAny, false, kStack, false, kW>(A, b + lane, b + lane < n, rays, hits, occl, skip);
   }
 }
 
