@@ -55,7 +55,6 @@ constexpr int kBinWords = 3 * kMaxBins * kBinVals;
 constexpr int kCntStride = 3 * kMaxBins;
 constexpr int kMaxRpt = 4;     // records per thread of a big node's chunk
 constexpr int kBigMin = 1024;  // big nodes have more triangles than this
-constexpr int kStageW = 256;   // records the global-memory warp split (oversized tasks) stages
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -159,20 +158,6 @@ __device__ __forceinline__ BinU binu_join(const BinU& x, const BinU& y) {
           fminf(x.a0, y.a0), fminf(x.a1, y.a1), fminf(x.a2, y.a2),
           fmaxf(x.b0, y.b0), fmaxf(x.b1, y.b1), fmaxf(x.b2, y.b2)};
 }
-__device__ __forceinline__ BinU binu_record(float4 lo, float4 hi) {
-  const float cx = centre(lo.x, hi.x), cy = centre(lo.y, hi.y), cz = centre(lo.z, hi.z);
-  return {1, lo.x, lo.y, lo.z, hi.x, hi.y, hi.z, cx, cy, cz, cx, cy, cz};
-}
-#define RT_BINU_SHFL(F, x, arg)                                                                               \
-  BinU {                                                                                                      \
-    F(kFull, (x).n, arg), F(kFull, (x).l0, arg), F(kFull, (x).l1, arg), F(kFull, (x).l2, arg),                \
-        F(kFull, (x).h0, arg), F(kFull, (x).h1, arg), F(kFull, (x).h2, arg), F(kFull, (x).a0, arg),           \
-        F(kFull, (x).a1, arg), F(kFull, (x).a2, arg), F(kFull, (x).b0, arg), F(kFull, (x).b1, arg),           \
-        F(kFull, (x).b2, arg)                                                                                 \
-  }
-__device__ __forceinline__ BinU binu_xor(const BinU& x, int o) { return RT_BINU_SHFL(__shfl_xor_sync, x, o); }
-#undef RT_BINU_SHFL
-
 // Decode a 13-word bin entry.
 __device__ __forceinline__ BinU binu_load(const unsigned* e) {
   const unsigned c = e[0];
@@ -222,13 +207,11 @@ __device__ __forceinline__ void bin_add_runs(int cell, const int* e, unsigned* b
   unsigned v[12];
 #pragma unroll
   for (int q = 0; q < 12; ++q) v[q] = c.v[q];
-#pragma unroll
+#pragma unroll 1
   for (int o = 1; o < 32; o <<= 1) {
+    const int from = max(lane - o, start);  // (idempotent: nothing to select past the run's start)
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-      const unsigned u = __shfl_up_sync(kFull, v[q], o);
-      if (lane - o >= start) v[q] = max(v[q], u);
-    }
+    for (int q = 0; q < 12; ++q) v[q] = max(v[q], __shfl_sync(kFull, v[q], from));
   }
   if (tail && cell >= 0) {
     const unsigned m = (unsigned)(lane - start + 1);
@@ -241,14 +224,6 @@ __device__ __forceinline__ void bin_add_runs(int cell, const int* e, unsigned* b
       if (cnt) atomicAdd(cnt + e[a], m);
     }
   }
-}
-
-// Add one record to bin entry `e` with plain shared-memory atomics (callers
-// spread the lanes over distant records, so lanes rarely share an entry).
-__device__ __forceinline__ void bin_add_plain(unsigned* e, const RecCodes& c) {
-  atomicAdd(e, 1u);
-#pragma unroll
-  for (int q = 0; q < 12; ++q) atomicMax(e + 1 + q, c.v[q]);
 }
 
 // ------------------------------------------------------------------ Eq. 2 evaluation
@@ -270,15 +245,18 @@ struct BinB {
   int n;
   float l0, l1, l2, h0, h1, h2;
 };
-__device__ __forceinline__ BinB binb_empty() { return {0, FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX}; }
 __device__ __forceinline__ BinB binb_join(const BinB& x, const BinB& y) {
   return {x.n + y.n,          fminf(x.l0, y.l0), fminf(x.l1, y.l1), fminf(x.l2, y.l2),
           fmaxf(x.h0, y.h0),  fmaxf(x.h1, y.h1), fmaxf(x.h2, y.h2)};
 }
-__device__ __forceinline__ BinB binb_load(const unsigned* e) {
-  const unsigned c = e[0];
-  if (c == 0) return binb_empty();
-  return {(int)c, uval(~e[1]), uval(~e[2]), uval(~e[3]), uval(e[4]), uval(e[5]), uval(e[6])};
+// The bin at e, the empty one unless `in`: loaded and selected without a
+// branch.  A lane that skips a load leaves its warp in two parts, and every
+// warp-wide operation after that meets at a slow rendezvous.
+__device__ __forceinline__ BinB binb_load(const unsigned* e, bool in) {
+  const unsigned c = e[0], w1 = e[1], w2 = e[2], w3 = e[3], w4 = e[4], w5 = e[5], w6 = e[6];
+  const bool f = in && c != 0;
+  return {f ? (int)c : 0,         f ? uval(~w1) : FLT_MAX,  f ? uval(~w2) : FLT_MAX, f ? uval(~w3) : FLT_MAX,
+          f ? uval(w4) : -FLT_MAX, f ? uval(w5) : -FLT_MAX, f ? uval(w6) : -FLT_MAX};
 }
 #define RT_BINB_SHFL(F, x, arg)                                                                            \
   BinB {                                                                                                   \
@@ -299,26 +277,27 @@ __device__ __forceinline__ BinB binb_load(const unsigned* e) {
 // kVals: words per bin (13, or 7 for bins of count and box only); kCentres:
 // gather the children's centre bounds (13-word bins only; otherwise the
 // caller derives the children's unions itself and only best.L.n is exact).
-template <int kVals, bool kCentres>
-__device__ __forceinline__ void eval_seg(const unsigned* bins0, int K, int n, int a0, int na, const CostP& cp,
-                                         Split& best) {
-  const int lane = threadIdx.x & 31;
-  const int g = lane / K, sl = lane - g * K;
-  const bool in = g < na;
+// eval_bins is the evaluation of bins held in registers (x: the lane's bin;
+// in: the lane holds one), eval_seg the one of bins in shared memory.
+template <bool kCentres>
+__device__ __forceinline__ void eval_bins(const BinB& x, const unsigned* e, bool in, int g, int sl, int K, int n, int a0,
+                                          const CostP& cp, Split& best) {
   const int a = a0 + (in ? g : 0);
-  const unsigned* e = bins0 + ((in ? g : 0) * K + sl) * kVals;
-  __syncwarp();
-  const BinB x = in ? binb_load(e) : binb_empty();
   BinB pre = x, suf = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    if (o >= K) break;
-    const BinB u = RT_BINB_SHFL(__shfl_up_sync, pre, o), d = RT_BINB_SHFL(__shfl_down_sync, suf, o);
-    if (sl >= o) pre = binb_join(pre, u);
-    if (sl + o < K) suf = binb_join(suf, d);
+  const int l0 = threadIdx.x & 31, first = l0 - sl, last = min(first + K - 1, 31);
+#pragma unroll 1
+  for (int o = 1; o < K; o <<= 1) {
+    // the boxes' unions are idempotent: a lane past its axis's end reads the
+    // end's own union and only the counts are selected
+    const int up = max(l0 - o, first), dn = min(l0 + o, last);
+    BinB u = RT_BINB_SHFL(__shfl_sync, pre, up), d = RT_BINB_SHFL(__shfl_sync, suf, dn);
+    u.n = sl >= o ? u.n : 0;
+    d.n = 0;  // (the right side's count is n minus the left's)
+    pre = binb_join(pre, u);
+    suf = binb_join(suf, d);
   }
   const BinB L = RT_BINB_SHFL(__shfl_up_sync, pre, 1);  // lane sl: bins 0 .. sl-1 of its axis
-  const BinB C = RT_BINB_SHFL(__shfl_sync, pre, min(g * K + K - 1, 31));
+  const BinB C = binb_join(L, suf);                     // the node (at sl >= 1, where a plane is)
   // Eq. 2 in every lane (a plane without records on both sides costs
   // infinity), then the lowest cost by two warp reductions: costs are >= +0
   // (alpha in [0, 1], t_i > 0, t_trav >= 0), so their bit patterns order as
@@ -340,7 +319,7 @@ __device__ __forceinline__ void eval_seg(const unsigned* bins0, int K, int n, in
     if (kCentres) {
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
-        const unsigned v = mine ? e[7 + q] : 0u;
+        const unsigned w = e[7 + q], v = mine ? w : 0u;
         lc[q] = __reduce_max_sync(kFull, sl < pl ? v : 0u);
         rc[q] = __reduce_max_sync(kFull, sl >= pl ? v : 0u);
       }
@@ -349,9 +328,20 @@ __device__ __forceinline__ void eval_seg(const unsigned* bins0, int K, int n, in
     best.cand = cand;
     best.L = {Lb.n, Lb.l0, Lb.l1, Lb.l2, Lb.h0, Lb.h1, Lb.h2,
               uval(~lc[0]), uval(~lc[1]), uval(~lc[2]), uval(lc[3]), uval(lc[4]), uval(lc[5])};
-    best.R = {Rb.n, Rb.l0, Rb.l1, Rb.l2, Rb.h0, Rb.h1, Rb.h2,
+    best.R = {n - Lb.n, Rb.l0, Rb.l1, Rb.l2, Rb.h0, Rb.h1, Rb.h2,
               uval(~rc[0]), uval(~rc[1]), uval(~rc[2]), uval(rc[3]), uval(rc[4]), uval(rc[5])};
   }
+}
+template <int kVals, bool kCentres>
+__device__ __forceinline__ void eval_seg(const unsigned* bins0, int K, int n, int a0, int na, const CostP& cp,
+                                         Split& best) {
+  const int lane = threadIdx.x & 31;
+  const int g = lane / K, sl = lane - g * K;
+  const bool in = g < na;
+  const unsigned* e = bins0 + ((in ? g : 0) * K + sl) * kVals;
+  __syncwarp();
+  const BinB x = binb_load(e, in);
+  eval_bins<kCentres>(x, e, in, g, sl, K, n, a0, cp, best);
 }
 #undef RT_BINB_SHFL
 
@@ -940,7 +930,7 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   // the barrier and read the choice from shared memory.  An axis without
   // extent has all records in bin 0 and yields no candidate.
   Split best;
-  if (warp < (3 * K <= 32 ? 1 : 3)) {
+  if (__any_sync(kFull, warp < (3 * K <= 32 ? 1 : 3))) {
     Split sp;
     split_none(sp);
     if (3 * K <= 32)
@@ -1160,7 +1150,7 @@ __device__ void top_emit(const BuildArgs& A, TopSmem& S, const TopTask& T, int s
           continue;
         }
       }
-      S.ptask[S.np++] = make_task(cb, cn, id, s, T.depth + 1, cu, par ^ 1);  // pools full: a warp takes it
+      S.ptask[S.np++] = make_task(cb, cn, id, s, T.depth + 1, cu, par ^ 1);  // pools full: a subtree task
     }
     if (S.created[0] || S.created[1])
       atomicAdd(&A.ctl->ti_pending, (S.created[0] ? nch0 : 0) + (S.created[1] ? nch1 : 0));
@@ -1241,7 +1231,10 @@ __device__ void top_loop(const BuildArgs& A, TopSmem& S, int epoch) {
 // subtree is the minimum of Eq. 2 over all splits of that order, evaluated
 // from warp scans of the records' boxes; ranges never move, so there is no
 // partition step, and all nodes of one level of the subtree are split
-// together (scans that stop at each node's bounds).
+// together (scans that stop at each node's bounds).  Nothing in it branches
+// by lane: where lanes part, every shuffle after that costs a rendezvous
+// (with branches in the scans, the node writes and the load of a short
+// node's records a node took 20k cycles of a busy SM, now 9k).
 struct Box6 {
   float l0, l1, l2, h0, h1, h2;
 };
@@ -1250,9 +1243,8 @@ __device__ __forceinline__ Box6 box_join(const Box6& a, const Box6& b) {
   return {fminf(a.l0, b.l0), fminf(a.l1, b.l1), fminf(a.l2, b.l2),
           fmaxf(a.h0, b.h0), fmaxf(a.h1, b.h1), fmaxf(a.h2, b.h2)};
 }
-__device__ __forceinline__ Box6 box_shfl_up(const Box6& a, int o) {
-  return {__shfl_up_sync(kFull, a.l0, o), __shfl_up_sync(kFull, a.l1, o), __shfl_up_sync(kFull, a.l2, o),
-          __shfl_up_sync(kFull, a.h0, o), __shfl_up_sync(kFull, a.h1, o), __shfl_up_sync(kFull, a.h2, o)};
+__device__ __forceinline__ Box6 box_sel(bool c, const Box6& a, const Box6& b) {
+  return {c ? a.l0 : b.l0, c ? a.l1 : b.l1, c ? a.l2 : b.l2, c ? a.h0 : b.h0, c ? a.h1 : b.h1, c ? a.h2 : b.h2};
 }
 __device__ __forceinline__ Box6 box_shfl_down(const Box6& a, int o) {
   return {__shfl_down_sync(kFull, a.l0, o), __shfl_down_sync(kFull, a.l1, o), __shfl_down_sync(kFull, a.l2, o),
@@ -1264,169 +1256,139 @@ __device__ __forceinline__ Box6 box_shfl(const Box6& a, int src) {
 }
 
 
-__device__ void micro_build(const BuildArgs& A, float4 rlo, float4 rhi, int n, int gbase, int parent, int side,
-                            int depth, int epoch, WarpStats& ws) {
+// Lane j: record j (box x) of the node of n records at gbase.  A lane is the
+// split position of at most one node of the subtree, so it keeps that node
+// (its own prefix and suffix unions are the children's boxes) and its
+// children's references, which it and its right neighbour know one level
+// later; all nodes are written together at the end.
+__device__ __forceinline__ void micro_build(const BuildArgs& A, const Box6& x, int n, int gbase, int parent, int side,
+                                            int depth, int epoch, WarpStats& ws) {
   const int lane = threadIdx.x & 31;
   // every lane follows the node its record belongs to: range [b, e), its
-  // parent, side and depth; lanes past n sit in empty ranges of their own
+  // parent and depth; lanes past n sit in empty ranges of their own
   const bool valid = lane < n;
   int b = valid ? 0 : lane, e = valid ? n : lane + 1;
-  int par = parent, sd = side, dep = depth;
-  const Box6 x = valid ? Box6{rlo.x, rlo.y, rlo.z, rhi.x, rhi.y, rhi.z} : box_empty();
-  int n_int = 0, n_leaf = 0, big = 0, deep = 0;  // per node, counted by its first lane
+  int par = parent, dep = depth;
+  // the node that this lane splits
+  Box6 nl = box_empty(), nr = box_empty();
+  int ob = 0, oe = 0, opar = 0, refl = 0, refr = 0;
+  bool own = false, fresh = false, root = false;
+#pragma unroll 1
   for (int level = 0; level < 32; ++level) {
     const bool active = valid && e - b > A.max_leaf;
     if (!__any_sync(kFull, active)) break;
+    const int width = (int)__reduce_max_sync(kFull, active ? (unsigned)(e - b) : 0u);
     // unions of the records from the start of the lane's node up to the lane
     // (ip) and from the lane to the node's end (is): scans that stop at the
     // node's bounds, all nodes of the level at once
     Box6 ip = x, is = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const Box6 u = box_shfl_up(ip, o), d = box_shfl_down(is, o);
-      if (lane - o >= b) ip = box_join(ip, u);
-      if (lane + o < e) is = box_join(is, d);
+#pragma unroll 1
+    for (int o = 1; o < width; o <<= 1) {
+      // a lane past the node's bound reads the bound's own union instead
+      // (unions are idempotent, so nothing has to be selected)
+      ip = box_join(ip, box_shfl(ip, max(lane - o, b)));
+      is = box_join(is, box_shfl(is, min(lane + o, e - 1)));
     }
-    const Box6 sufn = box_shfl_down(is, 1);    // records after the lane, within the node
-    const Box6 node = box_shfl(ip, e - 1);     // the whole node
-    const float3 clo = make_float3(node.l0, node.l1, node.l2), chi = make_float3(node.h0, node.h1, node.h2);
+    const Box6 sufn = box_shfl_down(is, 1);  // records after the lane, within the node
+    const Box6 node = box_shfl(ip, e - 1);   // the whole node
     // candidate: the lane is the last left record
-    float cost = INFINITY;
-    int cq = 1 << 20;
-    if (active && lane + 1 < e) {
-      const float c = eq2_cost(make_float3(ip.l0, ip.l1, ip.l2), make_float3(ip.h0, ip.h1, ip.h2), lane - b + 1,
-                               make_float3(sufn.l0, sufn.l1, sufn.l2), make_float3(sufn.h0, sufn.h1, sufn.h2),
-                               e - lane - 1, clo, chi, A.cp);
-      if (c < INFINITY) {
-        cost = c;
-        cq = lane;
-      }
-    }
-    // lowest cost of the node (ties: lowest position), found at its last lane
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float oc = __shfl_up_sync(kFull, cost, o);
-      const int oq = __shfl_up_sync(kFull, cq, o);
-      if (lane - o >= b && (oc < cost || (oc == cost && oq < cq))) {
-        cost = oc;
-        cq = oq;
-      }
-    }
-    const int wq = __shfl_sync(kFull, cq, e - 1);
-    const int q = !active ? lane : (wq < (1 << 20) ? wq : (b + e) / 2 - 1);  // no finite cost: middle
-    const int j = q + 1;                                                       // first record of the right child
-    const Box6 L = box_shfl(ip, q);
-    const Box6 R = box_shfl(is, min(j, 31));
-    if (active) {
-      const int id = gbase + q;
-      const int nl = j - b, nr = e - j;
-      const int rl = nl <= A.max_leaf ? leaf_ref(gbase + b, nl) : INT_MAX;
-      const int rr = nr <= A.max_leaf ? leaf_ref(gbase + j, nr) : INT_MAX;
-      if (lane == b) {
-        Node2 nd;
-        nd.a_lo = make_float4(L.l0, L.l1, L.l2, __int_as_float(rl));
-        nd.a_hi = make_float4(L.h0, L.h1, L.h2, __int_as_float(nl));
-        nd.b_lo = make_float4(R.l0, R.l1, R.l2, __int_as_float(rr));
-        nd.b_hi = make_float4(R.h0, R.h1, R.h2, __int_as_float(nr));
-        A.node2[id] = nd;
-        if (par < 0)
-          A.ctl->root_ref = id;
-        else if (par < A.n - 1)
-          *(sd == 0 ? &A.node2[par].a_lo.w : &A.node2[par].b_lo.w) = __int_as_float(id);
-        else
-          set_status(A.ctl, kStBadLink, 4);
-        A.link2[id] = make_int2(par, epoch);
-        ++n_int;
-        deep = max(deep, dep);
-        if (rl != INT_MAX) {
-          ++n_leaf;
-          big = max(big, nl);
-          deep = max(deep, dep + 1);
-        }
-        if (rr != INT_MAX) {
-          ++n_leaf;
-          big = max(big, nr);
-          deep = max(deep, dep + 1);
-        }
-      }
-      // follow the child holding this lane's record
-      if (lane < j) {
-        e = j;
-        sd = 0;
-      } else {
-        b = j;
-        sd = 1;
-      }
-      par = id;
-      ++dep;
+    const float c = eq2_cost(make_float3(ip.l0, ip.l1, ip.l2), make_float3(ip.h0, ip.h1, ip.h2), lane - b + 1,
+                             make_float3(sufn.l0, sufn.l1, sufn.l2), make_float3(sufn.h0, sufn.h1, sufn.h2),
+                             e - lane - 1, make_float3(node.l0, node.l1, node.l2),
+                             make_float3(node.h0, node.h1, node.h2), A.cp);
+    const bool ok = active && lane + 1 < e && c < INFINITY;
+    // lowest cost of the node (found at its last lane), and the lowest
+    // position that has it
+    const float cost = ok ? c : INFINITY;
+    float least = cost;
+#pragma unroll 1
+    for (int o = 1; o < width; o <<= 1) least = fminf(least, __shfl_sync(kFull, least, max(lane - o, b)));
+    least = __shfl_sync(kFull, least, e - 1);
+    const unsigned at = __ballot_sync(kFull, ok && cost == least) & (0xffffffffu >> (32 - e)) & (0xffffffffu << b);
+    const int q = !active ? lane : (at ? __ffs(at) - 1 : (b + e) / 2 - 1);  // no finite cost: middle
+    // the references of the nodes of this level, for those split on the last
+    const int ref = active ? gbase + q : leaf_ref(gbase + b, e - b), rref = __shfl_down_sync(kFull, ref, 1);
+    refl = fresh ? ref : refl;
+    refr = fresh ? rref : refr;
+    fresh = active && lane == q;
+    own = own || fresh;
+    root = root || (fresh && level == 0);
+    nl = box_sel(fresh, ip, nl);
+    nr = box_sel(fresh, sufn, nr);
+    ob = fresh ? b : ob;
+    oe = fresh ? e : oe;
+    opar = fresh ? par : opar;
+    // follow the child holding this lane's record
+    par = active ? gbase + q : par;
+    dep += active ? 1 : 0;
+    b = active && lane > q ? q + 1 : b;
+    e = active && lane <= q ? q + 1 : e;
+  }
+  const int ref = leaf_ref(gbase + b, e - b), rref = __shfl_down_sync(kFull, ref, 1);
+  refl = fresh ? ref : refl;
+  refr = fresh ? rref : refr;
+  // tree facts: every lane's last node is a leaf, one more leaf than nodes
+  const int nn = __popc(__ballot_sync(kFull, own));
+  ws.n_int += nn;
+  ws.n_leaf += nn ? nn + 1 : 0;
+  ws.big = max(ws.big, (int)__reduce_max_sync(kFull, valid ? (unsigned)(e - b) : 0u));
+  ws.deep = max(ws.deep, (int)__reduce_max_sync(kFull, valid ? (unsigned)dep : 0u));
+  if (own) {
+    const int id = gbase + lane;
+    Node2 nd;
+    nd.a_lo = make_float4(nl.l0, nl.l1, nl.l2, __int_as_float(refl));
+    nd.a_hi = make_float4(nl.h0, nl.h1, nl.h2, __int_as_float(lane + 1 - ob));
+    nd.b_lo = make_float4(nr.l0, nr.l1, nr.l2, __int_as_float(refr));
+    nd.b_hi = make_float4(nr.h0, nr.h1, nr.h2, __int_as_float(oe - lane - 1));
+    A.node2[id] = nd;
+    A.link2[id] = make_int2(opar, epoch);
+    if (root) {
+      if (parent < 0)
+        A.ctl->root_ref = id;
+      else if (parent < A.n - 1)
+        *(side == 0 ? &A.node2[parent].a_lo.w : &A.node2[parent].b_lo.w) = __int_as_float(id);
+      else
+        set_status(A.ctl, kStBadLink, 4);
     }
   }
-  ws.n_int += __reduce_add_sync(kFull, n_int);
-  ws.n_leaf += __reduce_add_sync(kFull, n_leaf);
-  ws.big = max(ws.big, (int)__reduce_max_sync(kFull, (unsigned)big));
-  ws.deep = max(ws.deep, (int)__reduce_max_sync(kFull, (unsigned)deep));
+  __syncwarp();
 }
 
-// A node of at most 32 records, record `lane` in registers (lo, hi): order
-// them by (Morton key, id) with a warp bitonic sort, write them to buffer 0
-// at gbegin in that order (the final order of their leaves) and build the
-// subtree.
-__device__ void micro_sort_build(const BuildArgs& A, float4 lo, float4 hi, int gbegin, int n, int parent, int side,
-                                 int depth, int epoch, WarpStats& ws) {
+// A node of 2 .. 32 records at src (shared memory, this warp's): order them
+// by (Morton key, id), each lane counting the records before its own, write
+// them to buffer 0 at gbegin in that order (the final order of their leaves)
+// and build the subtree.
+__device__ __forceinline__ void micro_sort_build(const BuildArgs& A, float4* src, int gbegin, int n, int parent,
+                                                 int side, int depth, int epoch, WarpStats& ws) {
   const int lane = threadIdx.x & 31;
-  unsigned long long key =
-      lane < n ? ((unsigned long long)__float_as_uint(hi.w) << 32) | (unsigned)__float_as_int(lo.w) : ~0ull;
-  int src = lane;
-  __syncwarp();
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      const unsigned long long ok = __shfl_xor_sync(kFull, key, jj);
-      const int os = __shfl_xor_sync(kFull, src, jj);
-      const bool up = (lane & k) == 0;
-      const bool lower = (lane & jj) == 0;
-      const bool take = (lower == up) ? (ok < key) : (ok > key);
-      if (take) {
-        key = ok;
-        src = os;
-      }
-    }
+  const int k = min(lane, n - 1);
+  float4 lo = src[2 * k], hi = src[2 * k + 1];
+  const unsigned key = __float_as_uint(hi.w), id = __float_as_uint(lo.w);
+  int rank = 0;
+#pragma unroll 4
+  for (int j = 0; j < n; ++j) {
+    const unsigned kj = __float_as_uint(src[2 * j + 1].w), ij = __float_as_uint(src[2 * j].w);
+    rank += (kj < key || (kj == key && ij < id)) ? 1 : 0;
   }
-  const float4 slo = make_float4(__shfl_sync(kFull, lo.x, src), __shfl_sync(kFull, lo.y, src),
-                                 __shfl_sync(kFull, lo.z, src), __shfl_sync(kFull, lo.w, src));
-  const float4 shi = make_float4(__shfl_sync(kFull, hi.x, src), __shfl_sync(kFull, hi.y, src),
-                                 __shfl_sync(kFull, hi.z, src), __shfl_sync(kFull, hi.w, src));
+  __syncwarp();
+  if (lane < n) {
+    src[2 * rank] = lo;
+    src[2 * rank + 1] = hi;
+  }
+  __syncwarp();
+  lo = src[2 * k];
+  hi = src[2 * k + 1];
   if (lane < n) {
     float4* p = A.rec[0] + 2 * ((size_t)gbegin + lane);
-    p[0] = slo;
-    p[1] = shi;
+    p[0] = lo;
+    p[1] = hi;
   }
-  if (__any_sync(kFull, n > A.max_leaf)) micro_build(A, slo, shi, n, gbegin, parent, side, depth, epoch, ws);
-}
-
-// micro_sort_build of a node whose records sit in global buffer `parity`.
-__device__ void micro_task(const BuildArgs& A, int begin, int n, int parity, int parent, int side, int depth,
-                           int epoch, WarpStats& ws) {
-  const int lane = threadIdx.x & 31;
-  float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-  if (lane < n) {
-    const float4* p = A.rec[parity] + 2 * ((size_t)begin + lane);
-    lo = __ldcg(p);
-    hi = __ldcg(p + 1);
-  }
-  micro_sort_build(A, lo, hi, begin, n, parent, side, depth, epoch, ws);
+  __syncwarp();
+  const Box6 x = box_sel(lane < n, Box6{lo.x, lo.y, lo.z, hi.x, hi.y, hi.z}, box_empty());
+  micro_build(A, x, n, gbegin, parent, side, depth, epoch, ws);
 }
 
 // ------------------------------------------------------------------ subtree queue
-// Claiming subtree tasks, and the split of tasks too large for a CTA's
-// shared memory (more than kSubMax records: a big node whose pools were
-// full, or any task when big = T / 4096 > 1024), done in global memory by
-// one warp until the part it keeps fits.
-struct MidWarp {
-  unsigned bins[kBinWords];
-  float4 stage[2 * kStageW];
-};
 // One thread takes the next queue slot and waits for it to be filled (the
 // other threads of the CTA wait at a barrier; nothing warp-synchronous runs
 // in this loop).  Returns false when the queue is drained (no big node and
@@ -1471,188 +1433,6 @@ __device__ bool claim_task(const BuildArgs& A, int epoch, Task& t) {
   }
 }
 
-// Split one node of more than 32 triangles with one warp (bin, Eq. 2, stable
-// partition), write it, and route its children: the larger internal child
-// becomes *cont, the other is queued, small ones are finished here.
-__device__ void mid_split(const BuildArgs& A, MidWarp& W, const Task& t, int epoch, WarpStats& ws, Task& cont,
-                          bool& have_cont) {
-  const int lane = threadIdx.x & 31;
-  const int K = A.K, K3 = 3 * K, n = t.count, par = t.pad & 1;
-  const float4* src = A.rec[par] + 2 * (size_t)t.begin;
-  float4* dst = A.rec[par ^ 1] + 2 * (size_t)t.begin;
-  const bool staged = n <= kStageW;
-  float cmin[3], scl[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    cmin[a] = t.clo[a];
-    scl[a] = bin_scale(t.clo[a], t.chi[a], K);
-  }
-  for (int w = lane; w < K3 * kBinVals; w += 32) W.bins[w] = 0u;
-  if (staged) {  // two records per lane in flight
-    for (int k0 = lane; k0 < n; k0 += 64) {
-      float4 v[4];
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-        if (k0 + 32 * u < n) {
-          v[2 * u] = __ldcg(src + 2 * (k0 + 32 * u));
-          v[2 * u + 1] = __ldcg(src + 2 * (k0 + 32 * u) + 1);
-        }
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-        if (k0 + 32 * u < n) {
-          W.stage[2 * (k0 + 32 * u)] = v[2 * u];
-          W.stage[2 * (k0 + 32 * u) + 1] = v[2 * u + 1];
-        }
-    }
-  }
-  __syncwarp();
-  // lane l bins records l*c .. l*c + c - 1: lanes work on distant records,
-  // which seldom share a bin, so plain atomics rarely collide
-  {
-    const int c = (n + 31) / 32;
-    for (int i = 0; i < c; ++i) {
-      const int k = lane * c + i;
-      if (k < n) {
-        const float4 lo = staged ? W.stage[2 * k] : __ldcg(src + 2 * k);
-        const float4 hi = staged ? W.stage[2 * k + 1] : __ldcg(src + 2 * k + 1);
-        const float cx = centre(lo.x, hi.x), cy = centre(lo.y, hi.y), cz = centre(lo.z, hi.z);
-        const RecCodes rc = rec_codes(lo, hi, cx, cy, cz);
-        bin_add_plain(W.bins + (0 * K + bin_of(cx, cmin[0], scl[0], K)) * kBinVals, rc);
-        bin_add_plain(W.bins + (1 * K + bin_of(cy, cmin[1], scl[1], K)) * kBinVals, rc);
-        bin_add_plain(W.bins + (2 * K + bin_of(cz, cmin[2], scl[2], K)) * kBinVals, rc);
-      }
-    }
-  }
-  __syncwarp();
-  Split best;
-  split_none(best);
-  if (3 * K <= 32) {  // all three axes in one pass
-    eval_axes(W.bins, K, n, 0, 3, A.cp, best);
-  } else if (2 * K <= 32) {  // x and y in one pass, then z
-    eval_axes(W.bins, K, n, 0, 2, A.cp, best);
-    if (__any_sync(kFull, scl[2] > 0.f)) eval_axis(W.bins, K, n, 2, A.cp, best);
-  } else {
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      if (__any_sync(kFull, scl[a] > 0.f)) eval_axis(W.bins, K, n, a, A.cp, best);
-  }
-  int axis, plane, nl;
-  if (best.cand != INT_MAX) {
-    axis = best.cand / (K - 1);
-    plane = 1 + best.cand % (K - 1);
-    nl = best.L.n;
-  } else {
-    axis = -1;
-    plane = 0;
-    nl = n / 2;
-  }
-  const float acmin = sel3(cmin[0], cmin[1], cmin[2], axis < 0 ? 0 : axis);
-  const float ascl = sel3(scl[0], scl[1], scl[2], axis < 0 ? 0 : axis);
-  // stable partition into the other buffer (child bounds by reduction when
-  // no plane was usable)
-  int lrun = 0, rrun = 0;
-  BinU accL = binu_empty(), accR = binu_empty();
-  for (int g = 0; __any_sync(kFull, g < n); g += 32) {
-    const int k = g + lane;
-    const bool valid = k < n;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (valid) {
-      if (staged) {
-        lo = W.stage[2 * k];
-        hi = W.stage[2 * k + 1];
-      } else {
-        lo = __ldcg(src + 2 * k);
-        hi = __ldcg(src + 2 * k + 1);
-      }
-    }
-    bool left = false;
-    if (valid) {
-      if (axis >= 0) {
-        const float cc = axis == 0 ? centre(lo.x, hi.x) : (axis == 1 ? centre(lo.y, hi.y) : centre(lo.z, hi.z));
-        left = bin_of(cc, acmin, ascl, K) < plane;
-      } else {
-        left = k < nl;
-      }
-    }
-    __syncwarp();
-    const unsigned bal = __ballot_sync(kFull, left);
-    const int rank = __popc(bal & ((1u << lane) - 1u));
-    const int dest = left ? lrun + rank : nl + rrun + (lane - rank);
-    if (valid && dest < n) {
-      dst[2 * dest] = lo;
-      dst[2 * dest + 1] = hi;
-      if (axis < 0) {
-        if (left)
-          accL = binu_join(accL, binu_record(lo, hi));
-        else
-          accR = binu_join(accR, binu_record(lo, hi));
-      }
-    }
-    const int tot = __popc(bal);
-    lrun += tot;
-    rrun += min(32, n - g) - tot;
-  }
-  BinU L = best.L, R = best.R;
-  if (__any_sync(kFull, axis < 0)) {
-    __syncwarp();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      accL = binu_join(accL, binu_xor(accL, o));
-      accR = binu_join(accR, binu_xor(accR, o));
-    }
-    L = accL;
-    R = accR;
-  }
-  if (lane == 0 && lrun != nl) set_status(A.ctl, kStBadSplit, 2);
-  __syncwarp();
-  const int nr = n - nl;
-  // leaves keep their records in buffer 0
-  if (par == 0) {
-    if (nl <= A.max_leaf)
-      for (int k = lane; k < 2 * nl; k += 32) A.rec[0][2 * (size_t)t.begin + k] = __ldcg(dst + k);
-    if (nr <= A.max_leaf)
-      for (int k = lane; k < 2 * nr; k += 32) A.rec[0][2 * ((size_t)t.begin + nl) + k] = __ldcg(dst + 2 * nl + k);
-  }
-  const int id = t.begin + nl - 1;
-  const int refl = nl <= A.max_leaf ? leaf_ref(t.begin, nl) : INT_MAX;
-  const int refr = nr <= A.max_leaf ? leaf_ref(t.begin + nl, nr) : INT_MAX;
-  if (lane == 0) write_node(A, id, t.parent, t.side, L, refl, nl, R, refr, nr, epoch);
-  ++ws.n_int;
-  const int leaves = (refl != INT_MAX) + (refr != INT_MAX);
-  ws.n_leaf += leaves;
-  if (refl != INT_MAX) ws.big = max(ws.big, nl);
-  if (refr != INT_MAX) ws.big = max(ws.big, nr);
-  ws.deep = max(ws.deep, leaves ? t.depth + 1 : t.depth);
-  // children: the larger one of more than 32 stays with this warp
-  L.n = nl;
-  R.n = nr;
-  const bool bigl = nl > kMicro, bigr = nr > kMicro;
-  const int keep = (bigl && bigr) ? (nl >= nr ? 0 : 1) : (bigl ? 0 : (bigr ? 1 : -1));
-  if (keep >= 0) {
-    cont = keep == 0 ? make_task(t.begin, nl, id, 0, t.depth + 1, L, par ^ 1)
-                     : make_task(t.begin + nl, nr, id, 1, t.depth + 1, R, par ^ 1);
-    have_cont = true;
-  }
-  if (lane == 0) {
-    Task out[3];
-    int k = 0;
-    if (bigl && bigr)  // the other big child
-      out[k++] = keep == 0 ? make_task(t.begin + nl, nr, id, 1, t.depth + 1, R, par ^ 1)
-                           : make_task(t.begin, nl, id, 0, t.depth + 1, L, par ^ 1);
-    // small subtrees go to idle warps while this one goes on down the tree
-    if (keep >= 0) {
-      if (nl > A.max_leaf && !bigl) out[k++] = make_task(t.begin, nl, id, 0, t.depth + 1, L, par ^ 1);
-      if (nr > A.max_leaf && !bigr) out[k++] = make_task(t.begin + nl, nr, id, 1, t.depth + 1, R, par ^ 1);
-    }
-    push_tasks(A, out, k, epoch);
-  }
-  __syncwarp();
-  if (keep < 0) {
-    if (nl > A.max_leaf) micro_task(A, t.begin, nl, par ^ 1, id, 0, t.depth + 1, epoch, ws);
-    if (nr > A.max_leaf) micro_task(A, t.begin + nl, nr, par ^ 1, id, 1, t.depth + 1, epoch, ws);
-  }
-}
-
 // ------------------------------------------------------------------ subtrees in shared memory
 // A CTA takes a task of at most kSubMax records, loads its records into
 // shared memory once and builds the subtree there.  Every node of more than
@@ -1664,6 +1444,8 @@ __device__ void mid_split(const BuildArgs& A, MidWarp& W, const Task& t, int epo
 // leave shared memory only as leaves, in their final order, into buffer 0.
 constexpr int kSubMax = 1024;            // records of a subtree built in shared memory
 constexpr int kMicroList = kSubMax / 2;  // nodes of at most 32 records (>= 2 each, disjoint)
+constexpr int kNodeThread = kBlock - 32;  // writes a CTA split's node: the last warp's first lane, so that the
+                                         // warps that evaluate Eq. 2 do not wait for its queue push
 constexpr int kBoxVals = 7;              // a subtree bin: count, box lo (complemented codes), box hi
 constexpr int kCtaBinWords = 3 * kMaxBins * kBoxVals + 4 * kBinVals;  // bins, then two sets of children's unions
 static_assert(kSubMax <= kBlock * 4, "a CTA partition keeps at most 4 records per thread");
@@ -1682,12 +1464,12 @@ struct SubSmem {
   int2 ml[kMicroList];  // nodes of at most 32: (parent, b | n << 10 | side << 16 | par << 17 | depth << 18)
   Task task;
   int red[kWarps];
-  int2 pick;  // the split Eq. 2 chose: candidate, records on the left
+  int2 pick[3];     // the split Eq. 2 chose on each group of axes: candidate, records on the left
+  float pcost[3];
   int mord[32];  // the order in which the warps take the small nodes (largest first)
-  float4 pbox[3];  // and the boxes of its children (left lo, hi; right lo, hi)
+  float4 pbox[3][3];  // and the boxes of its children (left lo, hi; right lo, hi)
   int nm, mnext, got;
 };
-static_assert(sizeof(MidWarp) <= sizeof(float4) * 2 * 2 * kSubMax, "a warp's global-memory split state fits");
 
 __device__ __forceinline__ SubNode sub_node(int b, int n, int parent, int side, int depth, int par, const BinU& u) {
   SubNode x;
@@ -1721,12 +1503,17 @@ __device__ __forceinline__ void flush_box(unsigned* e, const unsigned* acc) {
 #pragma unroll
   for (int q = 1; q < kBoxVals; ++q) atomicMax(e + q, acc[q]);
 }
+template <bool kGlobal>
+__device__ __forceinline__ float4 rec_load(const float4* p) {
+  return kGlobal ? __ldcg(p) : *p;
+}
+template <bool kGlobal>
 __device__ __forceinline__ void bin_run(unsigned* bins, const float4* src, int k0, int k1, int K, const float* cmin,
                                         const float* scl) {
   int key[3] = {-1, -1, -1};
   unsigned acc[3][kBoxVals];
   for (int k = k0; k < k1; ++k) {
-    const float4 lo = src[2 * k], hi = src[2 * k + 1];
+    const float4 lo = rec_load<kGlobal>(src + 2 * k), hi = rec_load<kGlobal>(src + 2 * k + 1);
     const unsigned c6[6] = {~ucode(lo.x), ~ucode(lo.y), ~ucode(lo.z), ucode(hi.x), ucode(hi.y), ucode(hi.z)};
     const float cc[3] = {centre(lo.x, hi.x), centre(lo.y, hi.y), centre(lo.z, hi.z)};
 #pragma unroll
@@ -1750,86 +1537,98 @@ __device__ __forceinline__ void bin_run(unsigned* bins, const float4* src, int k
     if (key[a] >= 0) flush_box(bins + (a * K + key[a]) * kBoxVals, acc[a]);
 }
 
-// Eq. 2 over the 7-word bins of all three axes (as many axes per warp pass
-// as 32 lanes hold).  Only best.cand and best.L.n are used afterwards.
-__device__ __forceinline__ void eval_box(const unsigned* bins, int K, int n, const float* scl, const CostP& cp,
-                                         Split& best) {
-  for (int g = 0; g < 3;) {
-    const int m = min(3 - g, 32 / K);
-    if (m >= 2 || __any_sync(kFull, scl[g] > 0.f))
-      eval_seg<kBoxVals, false>(bins + g * K * kBoxVals, K, n, g, m, cp, best);
-    g += m;
-  }
-}
-
-// A child's union (count, box, centre bounds) accumulated over records: 13
-// words in bin order (count, then the codes of a record).
-__device__ __forceinline__ void acc13_add(unsigned* v, const RecCodes& c) {
-  v[0] += 1u;
-#pragma unroll
-  for (int q = 0; q < 12; ++q) v[1 + q] = max(v[1 + q], c.v[q]);
-}
+// A warp's union of its lanes' 13 words (count, then the codes of a record).
 __device__ __forceinline__ void acc13_warp(unsigned* v) {
   v[0] = __reduce_add_sync(kFull, v[0]);
 #pragma unroll
   for (int q = 1; q < kBinVals; ++q) v[q] = __reduce_max_sync(kFull, v[q]);
 }
 
-// Copy a leaf's records from shared memory to buffer 0 (its final place).
+// Copy a leaf's records from shared memory (or buffer 1) to buffer 0 (their
+// final place).
+template <bool kGlobal>
 __device__ __forceinline__ void leaf_out(const BuildArgs& A, const float4* src, int gpos, int n, int t0, int nt) {
-  for (int k = t0; k < 2 * n; k += nt) A.rec[0][2 * (size_t)gpos + k] = src[k];
+  for (int k = t0; k < 2 * n; k += nt) A.rec[0][2 * (size_t)gpos + k] = rec_load<kGlobal>(src + k);
 }
 
 
 // Split node X of the subtree with the whole CTA (split `it` of the task's
 // chain): bins (count and box) in one shared array, each thread binning a
 // run of records (thread (w, l) takes run l * 8 + w, so the lanes of a warp
-// work far apart); Eq. 2 evaluated by warp 0, its choice read by all from
-// shared memory (one warp's shuffles instead of eight); stable partition by
-// a block scan, which also gathers both children's unions (into one of two
+// work far apart); Eq. 2 evaluated by one to three warps, the axes divided
+// among them, their choices read by all from shared memory; stable partition
+// by a block scan, which also gathers both children's unions (into one of two
 // sets, alternating with `it`) and clears the bins and the other set for
-// the next split.  Thread 0 writes the node and routes the other children:
+// the next split.  One thread writes the node and routes the other children:
 // the smaller one of more than 32 records goes to the device queue, those
 // of at most 32 to the small-node list.  If the larger child has more than
 // 32 records, every thread makes it X (true) and goes on without a barrier.
-__device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, int gbegin, int tdepth, int epoch,
-                          WarpStats& ws) {
+// Bound by the latency of its dependent steps: a split of 33 .. 64 records
+// takes 7.0k cycles (11.9k when one warp evaluated all axes, with branches
+// that left it in two parts), of which Eq. 2 2.7k (6.6k).
+//
+// kGlobal: the same split of a node too large for shared memory (more than
+// kSubMax records: big = T / 4096 of a scene of more than 4M triangles, or a
+// big node whose pools were full), its records in global buffer X.par, the
+// children's in the other; both children that are not leaves become tasks
+// except the larger one, which is X again whatever its size (true while it
+// is still too large).
+template <bool kGlobal>
+__device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, int gbegin, int tdepth,
+                                          int epoch, WarpStats& ws) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = A.K, n = X.n, p = X.par;
   const int nbw = 3 * K * kBoxVals;
   unsigned* cb = S.bins;  // zero on entry
   unsigned* cu = cb + nbw + (it & 1) * 2 * kBinVals;  // the children's unions, 2 x 13 words (zero on entry)
   unsigned* cu_next = cb + nbw + ((it + 1) & 1) * 2 * kBinVals;
-  const float4* src = S.rec[p] + 2 * X.b;
-  float4* dst = S.rec[p ^ 1] + 2 * X.b;
+  const float4* src = kGlobal ? A.rec[p] + 2 * ((size_t)gbegin + X.b) : S.rec[p] + 2 * X.b;
+  float4* dst = kGlobal ? A.rec[p ^ 1] + 2 * ((size_t)gbegin + X.b) : S.rec[p ^ 1] + 2 * X.b;
   float cmin[3], scl[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     cmin[a] = X.clo[a];
     scl[a] = bin_scale(X.clo[a], X.chi[a], K);
   }
-  // thread t owns records [t c, t c + c), c <= 4, for the partition; runs
-  // for the bins use the spread order
+  // thread t owns records [t c, t c + c) for the partition; runs for the
+  // bins use the spread order
   const int c = (n + kBlock - 1) / kBlock;
   {
     const int r = lane * kWarps + warp, k0 = min(r * c, n), k1 = min(k0 + c, n);
-    bin_run(cb, src, k0, k1, K, cmin, scl);
+    bin_run<kGlobal>(cb, src, k0, k1, K, cmin, scl);
   }
   __syncthreads();
-  if (warp == 0) {  // one warp evaluates Eq. 2 (the others wait at the barrier)
+  // Eq. 2: as many axes per warp as 32 lanes hold, warp g the g-th group of
+  // them (the others wait at the barrier); every thread then takes the lower
+  // cost, the lower candidate among equal costs
+  const int apw = min(3, 32 / K), ngr = (2 + apw) / apw;
+  if (__any_sync(kFull, warp < ngr)) {
+    const int a0 = warp * apw, m = min(3 - a0, apw);
     Split best;
     split_none(best);
-    eval_box(cb, K, n, scl, A.cp, best);
+    if (m >= 2 || __any_sync(kFull, sel3(scl[0], scl[1], scl[2], a0) > 0.f))
+      eval_seg<kBoxVals, false>(cb + a0 * K * kBoxVals, K, n, a0, m, A.cp, best);
     if (lane == 0) {
-      S.pick = make_int2(best.cand, best.L.n);
+      S.pcost[warp] = best.cost;
+      S.pick[warp] = make_int2(best.cand, best.L.n);
       // both children's boxes: the unions of the bins' boxes on each side
-      S.pbox[0] = make_float4(best.L.l0, best.L.l1, best.L.l2, best.L.h0);
-      S.pbox[1] = make_float4(best.L.h1, best.L.h2, best.R.l0, best.R.l1);
-      S.pbox[2] = make_float4(best.R.l2, best.R.h0, best.R.h1, best.R.h2);
+      S.pbox[warp][0] = make_float4(best.L.l0, best.L.l1, best.L.l2, best.L.h0);
+      S.pbox[warp][1] = make_float4(best.L.h1, best.L.h2, best.R.l0, best.R.l1);
+      S.pbox[warp][2] = make_float4(best.R.l2, best.R.h0, best.R.h1, best.R.h2);
     }
   }
   __syncthreads();
-  const int2 pick = S.pick;
+  int win = 0;
+  int2 pick = S.pick[0];
+  float pcost = S.pcost[0];
+  for (int g = 1; g < ngr; ++g) {
+    const float c = S.pcost[g];
+    const int2 q = S.pick[g];
+    const bool lower = c < pcost || (c == pcost && q.x < pick.x);
+    win = lower ? g : win;
+    pick = lower ? q : pick;
+    pcost = lower ? c : pcost;
+  }
   int axis, plane, nl;
   if (pick.x != INT_MAX) {
     axis = pick.x / (K - 1);
@@ -1843,27 +1642,16 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
   const float acmin = sel3(cmin[0], cmin[1], cmin[2], axis < 0 ? 0 : axis);
   const float ascl = sel3(scl[0], scl[1], scl[2], axis < 0 ? 0 : axis);
   const int k0 = min(tid * c, n);
-  float4 rl[4], rh[4];
-  unsigned fl = 0;
+  const int k1 = min(k0 + c, n);
+  auto goes_left = [&](int k) {
+    if (axis < 0) return k < nl;
+    const float* q = reinterpret_cast<const float*>(src + 2 * k) + axis;
+    const float cc = kGlobal ? centre(__ldcg(q), __ldcg(q + 4)) : centre(q[0], q[4]);
+    return bin_of(cc, acmin, ascl, K) < plane;
+  };
   int cnt = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = k0 + i;
-    if (i < c && k < n) {
-      rl[i] = src[2 * k];
-      rh[i] = src[2 * k + 1];
-      bool left;
-      if (axis >= 0) {
-        const float cc = axis == 0 ? centre(rl[i].x, rh[i].x)
-                                   : (axis == 1 ? centre(rl[i].y, rh[i].y) : centre(rl[i].z, rh[i].z));
-        left = bin_of(cc, acmin, ascl, K) < plane;
-      } else {
-        left = k < nl;
-      }
-      fl |= (unsigned)left << i;
-      cnt += left;
-    }
-  }
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) cnt += goes_left(k);
   int inc = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -1895,27 +1683,31 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
   unsigned ua[kBinVals], ub[kBinVals];
 #pragma unroll
   for (int q = 0; q < kBinVals; ++q) ua[q] = ub[q] = 0u;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = k0 + i;
-    if (i < c && k < n) {
-      const bool left = (fl >> i) & 1u;
-      const int d = left ? lb++ : nl + rb++;
-      if (d < n) {
-        if ((left ? 0 : 1) == ex) {
-          __stcg(gx + 2 * d, rl[i]);
-          __stcg(gx + 2 * d + 1, rh[i]);
-        } else {
-          dst[2 * d] = rl[i];
-          dst[2 * d + 1] = rh[i];
-        }
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    const float4 rl = rec_load<kGlobal>(src + 2 * k), rh = rec_load<kGlobal>(src + 2 * k + 1);
+    const bool left = goes_left(k);
+    const int d = left ? lb++ : nl + rb++;
+    if (d < n) {
+      if (kGlobal) {
+        __stcg(dst + 2 * d, rl);
+        __stcg(dst + 2 * d + 1, rh);
+      } else if ((left ? 0 : 1) == ex) {
+        __stcg(gx + 2 * d, rl);
+        __stcg(gx + 2 * d + 1, rh);
+      } else {
+        dst[2 * d] = rl;
+        dst[2 * d + 1] = rh;
       }
-      const RecCodes rc =
-          rec_codes(rl[i], rh[i], centre(rl[i].x, rh[i].x), centre(rl[i].y, rh[i].y), centre(rl[i].z, rh[i].z));
-      if (left)
-        acc13_add(ua, rc);
-      else
-        acc13_add(ub, rc);
+    }
+    const RecCodes rc = rec_codes(rl, rh, centre(rl.x, rh.x), centre(rl.y, rh.y), centre(rl.z, rh.z));
+    const unsigned ml = left ? 0xffffffffu : 0u;  // the codes of the other side count as empty (0)
+    ua[0] += left ? 1u : 0u;
+    ub[0] += left ? 0u : 1u;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+      ua[1 + q] = max(ua[1 + q], rc.v[q] & ml);
+      ub[1 + q] = max(ub[1 + q], rc.v[q] & ~ml);
     }
   }
   // the children's unions: with a plane, count and box are known (Eq. 2's
@@ -1950,7 +1742,7 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
   __syncthreads();
   BinU L, R;
   if (axis >= 0) {
-    const float4 b0 = S.pbox[0], b1 = S.pbox[1], b2 = S.pbox[2];
+    const float4 b0 = S.pbox[win][0], b1 = S.pbox[win][1], b2 = S.pbox[win][2];
     L = {nl, b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, uval(~cu[7]), uval(~cu[8]), uval(~cu[9]), uval(cu[10]),
          uval(cu[11]), uval(cu[12])};
     R = {n - nl, b1.z, b1.w, b2.x, b2.y, b2.z, b2.w, uval(~cu[kBinVals + 7]), uval(~cu[kBinVals + 8]),
@@ -1960,10 +1752,12 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
     R = binu_load(cu + kBinVals);
   }
   const bool leafl = nl <= A.max_leaf, leafr = nr <= A.max_leaf;
-  if (leafl) leaf_out(A, dst, gbegin + X.b, nl, tid, kBlock);
-  if (leafr) leaf_out(A, dst + 2 * nl, gbegin + X.b + nl, nr, tid, kBlock);
+  if (!kGlobal || p == 0) {  // (a leaf of a global split from buffer 1 is in buffer 0 already)
+    if (leafl) leaf_out<kGlobal>(A, dst, gbegin + X.b, nl, tid, kBlock);
+    if (leafr) leaf_out<kGlobal>(A, dst + 2 * nl, gbegin + X.b + nl, nr, tid, kBlock);
+  }
   const int id = gbegin + X.b + nl - 1;
-  if (tid == 0) {
+  if (tid == kNodeThread) {
     if (total != nl) set_status(A.ctl, kStBadSplit, 6);
     write_node(A, id, X.parent, X.side, L, leafl ? leaf_ref(gbegin + X.b, nl) : INT_MAX, nl, R,
                leafr ? leaf_ref(gbegin + X.b + nl, nr) : INT_MAX, nr, epoch);
@@ -1972,7 +1766,9 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
     for (int s = 0; s < 2; ++s) {
       const int cn = s ? nr : nl, b = X.b + (s ? nl : 0);
       if (cn <= A.max_leaf) continue;
-      if (s == ex) {
+      if (kGlobal) {
+        if (s != keep) push_task(A, make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, p ^ 1), epoch);
+      } else if (s == ex) {
         // the records written to buffer 1 by every thread are ordered before
         // this thread by the barrier; push_task's release store publishes them
         push_task(A, make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, 1), epoch);
@@ -1985,27 +1781,28 @@ __device__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNode& X, int it, in
     }
   }
   // every thread takes the kept child from the unions it read (no barrier:
-  // thread 0's node write and release fence overlap the next split's
+  // the node thread's write and release fence overlap the next split's
   // binning, which reads only the kept child's records)
-  if ((keep ? nr : nl) <= kMicro) return false;
+  if (!kGlobal && (keep ? nr : nl) <= kMicro) return false;
   X = sub_node(X.b + (keep ? nl : 0), keep ? nr : nl, id, keep, X.depth + 1, p ^ 1, keep ? R : L);
-  return true;
+  return !kGlobal || X.n > kSubMax;
 }
 
 // The warps finish the collected nodes of at most 32 records, one node per
 // warp at a time (no node is added any more).
-__device__ void micro_phase(const BuildArgs& A, SubSmem& S, int gbegin, int tdepth, int epoch, WarpStats& ws) {
+__device__ __forceinline__ void micro_phase(const BuildArgs& A, SubSmem& S, int gbegin, int tdepth, int epoch,
+                                            WarpStats& ws) {
   const int lane = threadIdx.x & 31;
   const int nm = S.nm;
   // more nodes than warps (up to 32): warp 0 orders them largest first, so
   // that the last round of builds holds the quickest ones
   const bool order = nm > kWarps && nm <= 32;
   if (order) {
-    if (threadIdx.x < 32) {
+    if (__any_sync(kFull, threadIdx.x < 32)) {
       unsigned key = lane < nm ? ((unsigned)(63 - ((S.ml[lane].y >> 10) & 63)) << 8) | (unsigned)lane : 0xffffffffu;
-#pragma unroll
+#pragma unroll 1
       for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
+#pragma unroll 1
         for (int jj = k >> 1; jj > 0; jj >>= 1) {
           const unsigned ok = __shfl_xor_sync(kFull, key, jj);
           const bool up = (lane & k) == 0, lower = (lane & jj) == 0;
@@ -2023,14 +1820,27 @@ __device__ void micro_phase(const BuildArgs& A, SubSmem& S, int gbegin, int tdep
     if (i >= nm) break;
     const int2 m = S.ml[order ? S.mord[i] : i];
     const int f = m.y;
-    const int b = f & 1023, n = (f >> 10) & 63, side = (f >> 16) & 1, par = (f >> 17) & 1, dep = f >> 18;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (lane < n) {
-      lo = S.rec[par][2 * (b + lane)];
-      hi = S.rec[par][2 * (b + lane) + 1];
-    }
-    micro_sort_build(A, lo, hi, gbegin + b, n, m.x, side, tdepth + dep, epoch, ws);
+    const int b = f & 1023, n = __shfl_sync(kFull, (f >> 10) & 63, 0), side = (f >> 16) & 1, par = (f >> 17) & 1,
+              dep = f >> 18;
+    micro_sort_build(A, S.rec[par] + 2 * b, gbegin + b, n, m.x, side, tdepth + dep, epoch, ws);
   }
+}
+
+// Task t as a node of its own range, its records in buffer par.
+__device__ __forceinline__ SubNode task_node(const Task& t, int par) {
+  SubNode X;
+  X.b = 0;
+  X.n = t.count;
+  X.parent = t.parent;
+  X.side = t.side;
+  X.depth = t.depth;
+  X.par = par;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    X.clo[a] = t.clo[a];
+    X.chi[a] = t.chi[a];
+  }
+  return X;
 }
 
 // Build the subtree of task t (max_leaf < t.count <= kSubMax) in shared
@@ -2042,39 +1852,27 @@ __device__ void sub_tree(const BuildArgs& A, SubSmem& S, const Task& t, int epoc
   for (int k = tid; k < 2 * n; k += kBlock) S.rec[0][k] = __ldcg(g + k);
   // the first split's bins and unions start at zero
   for (int w = tid; w < kCtaBinWords; w += kBlock) S.bins[w] = 0u;
-  if (tid == 0) {
+  __syncthreads();
+  if (tid == kNodeThread) {
     S.nm = 0;
     S.mnext = 0;
     if (n <= kMicro) S.ml[S.nm++] = micro_pack(0, n, t.parent, t.side, 0, 0);
   }
-  __syncthreads();
   if (n > kMicro) {  // the chain of larger children, split by the whole CTA
-    SubNode X;
-    X.b = 0;
-    X.n = n;
-    X.parent = t.parent;
-    X.side = t.side;
-    X.depth = t.depth;
-    X.par = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      X.clo[a] = t.clo[a];
-      X.chi[a] = t.chi[a];
+    SubNode X = task_node(t, 0);
+    for (int it = 0; cta_split<false>(A, S, X, it, t.begin, t.depth, epoch, ws); ++it) {
     }
-    for (int it = 0; cta_split(A, S, X, it, t.begin, t.depth, epoch, ws); ++it) {
-    }
-    __syncthreads();  // thread 0's last additions to the small-node list
   }
+  __syncthreads();  // the node thread's last additions to the small-node list
   micro_phase(A, S, t.begin, t.depth, epoch, ws);
   __syncthreads();
 }
 
 // The subtree role of every CTA: take a task from the queue, build its
 // subtree (tasks of more than kSubMax records are first split in global
-// memory by one warp, down to a part that fits), repeat until the queue is
-// drained.
+// memory, down to a part that fits), repeat until the queue is drained.
 __device__ void sub_loop(const BuildArgs& A, SubSmem& S, int epoch) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   WarpStats ws{0, 0, 0, 0};
   for (;;) {
     if (tid == 0) S.got = claim_task(A, epoch, S.task);
@@ -2093,28 +1891,26 @@ __device__ void sub_loop(const BuildArgs& A, SubSmem& S, int epoch) {
           A.rec[0][2 * (size_t)t.begin + k] = __ldcg(A.rec[1] + 2 * (size_t)t.begin + k);
     } else {
       if (t.count > kSubMax) {
-        if (warp == 0) {
-          MidWarp& W = *reinterpret_cast<MidWarp*>(&S.rec[0][0]);
-          Task cur = t;
-          bool more = true;
-          while (more && cur.count > kSubMax) {
-            Task nx;
-            more = false;
-            mid_split(A, W, cur, epoch, ws, nx, more);
-            if (more) cur = nx;
-          }
-          if (lane == 0) {
-            S.got = more;
-            S.task = cur;
-          }
+        // split in global memory, down to a part that fits
+        for (int w = tid; w < kCtaBinWords; w += kBlock) S.bins[w] = 0u;
+        __syncthreads();
+        SubNode X = task_node(t, par);
+        for (int it = 0; cta_split<true>(A, S, X, it, t.begin, t.depth, epoch, ws); ++it) {
+        }
+        t.begin += X.b;
+        t.count = X.n;
+        t.parent = X.parent;
+        t.side = X.side;
+        t.depth = X.depth;
+        t.pad = X.par;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          t.clo[a] = X.clo[a];
+          t.chi[a] = X.chi[a];
         }
         __syncthreads();
-        t = S.task;
-        const bool more = S.got;
-        __syncthreads();
-        if (!more) t.count = 0;
       }
-      if (t.count > 0) sub_tree(A, S, t, epoch, ws);
+      sub_tree(A, S, t, epoch, ws);
     }
     __syncthreads();
     // the pushes of this task counted first, so this never reads zero early
@@ -2445,7 +2241,7 @@ BuildGeom build_geometry(int64_t n, int nsm) {
   rpt = std::min<int64_t>(std::max<int64_t>(rpt, 1), kMaxRpt);
   g.rpt = (int)rpt;
   g.chunk = kBlock * g.rpt;
-  // Pools of one build (a full pool sends further big nodes to the warps,
+  // Pools of one build (a full pool sends further big nodes to the subtree queue,
   // slower but correct).  Big nodes of one depth are disjoint, so there are at
   // most T / big of them per depth; 16 depths' worth covers the uneven trees
   // of alpha < 1.  Chunk counts: a big node reserves its chunks + 2 for its
