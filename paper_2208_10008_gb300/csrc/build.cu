@@ -24,6 +24,8 @@
 //                 most 32 finished by single warps in registers over the
 //                 Morton order of their records.  No CTA waits for another
 //                 except for work to appear (bounded waits).
+//   k_small       (large scenes) the subtrees of the nodes of at most 64 or 128
+//                 records that k_split then leaves, a warp each
 //   k_post        4-wide traversal nodes (greedy by surface area), stored at the
 //                 id of their binary root; triangles in leaf order
 //
@@ -245,6 +247,7 @@ struct BinB {
   int n;
   float l0, l1, l2, h0, h1, h2;
 };
+__device__ __forceinline__ BinB binb_empty() { return {0, FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX}; }
 __device__ __forceinline__ BinB binb_join(const BinB& x, const BinB& y) {
   return {x.n + y.n,          fminf(x.l0, y.l0), fminf(x.l1, y.l1), fminf(x.l2, y.l2),
           fmaxf(x.h0, y.h0),  fmaxf(x.h1, y.h1), fmaxf(x.h2, y.h2)};
@@ -343,6 +346,7 @@ __device__ __forceinline__ void eval_seg(const unsigned* bins0, int K, int n, in
   const BinB x = binb_load(e, in);
   eval_bins<kCentres>(x, e, in, g, sl, K, n, a0, cp, best);
 }
+__device__ __forceinline__ BinB binb_xor(const BinB& x, int o) { return RT_BINB_SHFL(__shfl_xor_sync, x, o); }
 #undef RT_BINB_SHFL
 
 __device__ __forceinline__ void eval_axis(const unsigned* bins, int K, int n, int a, const CostP& cp, Split& best) {
@@ -382,6 +386,7 @@ struct BuildArgs {
   int n, K, max_leaf;  // n: records in this build
   int n_all;           // triangles in the scene (input ids are below it)
   int big, chunk, rpt, cap_t, cap_c, qa_cap, top_ctas;
+  int wsm;             // nodes of up to this many records go to k_small (0: none do)
   int spin_limit;                    // polls without progress before a wait gives up
   int phantom_tasks, phantom_items;  // test hooks: pending work that never comes
   CostP cp;
@@ -441,6 +446,18 @@ __device__ void push_tasks(const BuildArgs& A, const Task* t, int k, int epoch) 
   atomicAdd(&A.ctl->qa_pending, k);
   for (int i = 0; i < k; ++i) A.qa[s + i] = t[i];
   for (int i = 0; i < k; ++i) st_release(&A.qa_ready[s + i], epoch);
+}
+
+// Hand a node of at most A.wsm records to k_small (one thread): its list
+// grows down from the end of the task array (a tree node is in one of the
+// two at most, so they never meet in a valid tree).
+__device__ void push_small(const BuildArgs& A, const Task& t) {
+  const int i = atomicAdd(&A.ctl->sq_count, 1);
+  if (i >= A.qa_cap - ld_volatile(&A.ctl->qa_tail)) {
+    set_status(A.ctl, kStQueueOverflow, 6);
+    return;
+  }
+  A.qa[A.qa_cap - 1 - i] = t;
 }
 
 __device__ __forceinline__ Task make_task(int begin, int count, int parent, int side, int depth, const BinU& u,
@@ -1161,7 +1178,16 @@ __device__ void top_emit(const BuildArgs& A, TopSmem& S, const TopTask& T, int s
   // count); meanwhile a thread of warp 1 hands the subtree-sized children to
   // the subtree queue (one reservation, release stores), so that neither
   // publication waits for the other's fence
-  if (tid == 32 && S.np > 0) push_tasks(A, S.ptask, S.np, epoch);
+  if (tid == 32 && S.np > 0) {
+    int k = 0;
+    for (int i = 0; i < S.np; ++i) {
+      if (A.wsm && S.ptask[i].count <= A.wsm && S.ptask[i].count > A.max_leaf)
+        push_small(A, S.ptask[i]);
+      else
+        S.ptask[k++] = S.ptask[i];
+    }
+    push_tasks(A, S.ptask, k, epoch);
+  }
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     if (!S.created[s]) continue;
@@ -1443,6 +1469,7 @@ __device__ bool claim_task(const BuildArgs& A, int epoch, Task& t) {
 // and finished at the end by the warps in parallel, in registers.  Records
 // leave shared memory only as leaves, in their final order, into buffer 0.
 constexpr int kSubMax = 1024;            // records of a subtree built in shared memory
+constexpr int kWarpMax = 128;            // largest node that a warp of k_small takes (4 records per lane)
 constexpr int kMicroList = kSubMax / 2;  // nodes of at most 32 records (>= 2 each, disjoint)
 constexpr int kNodeThread = kBlock - 32;  // writes a CTA split's node: the last warp's first lane, so that the
                                          // warps that evaluate Eq. 2 do not wait for its queue push
@@ -1678,7 +1705,13 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
   // buffer 1 here instead of to shared memory
   const int nr = n - nl;
   const int keep = nl >= nr ? 0 : 1;
-  const int ex = (keep == 0 ? nr : nl) > kMicro ? 1 - keep : -1;
+  const int lim = kGlobal ? kSubMax : (A.wsm ? A.wsm : kMicro);  // the chain ends at nodes of this size
+  bool ex[2];  // children that leave shared memory: the smaller one, to the queue, and k_small's nodes
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int cn = s ? nr : nl;
+    ex[s] = cn > lim ? s != keep : A.wsm && cn > A.max_leaf;
+  }
   float4* gx = A.rec[1] + 2 * ((size_t)gbegin + X.b);
   unsigned ua[kBinVals], ub[kBinVals];
 #pragma unroll
@@ -1692,7 +1725,7 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
       if (kGlobal) {
         __stcg(dst + 2 * d, rl);
         __stcg(dst + 2 * d + 1, rh);
-      } else if ((left ? 0 : 1) == ex) {
+      } else if (left ? ex[0] : ex[1]) {
         __stcg(gx + 2 * d, rl);
         __stcg(gx + 2 * d + 1, rh);
       } else {
@@ -1766,9 +1799,17 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
     for (int s = 0; s < 2; ++s) {
       const int cn = s ? nr : nl, b = X.b + (s ? nl : 0);
       if (cn <= A.max_leaf) continue;
+      const bool small = A.wsm && cn <= A.wsm;
       if (kGlobal) {
-        if (s != keep) push_task(A, make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, p ^ 1), epoch);
-      } else if (s == ex) {
+        const Task c = make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, p ^ 1);
+        if (s == keep) continue;
+        if (small)
+          push_small(A, c);
+        else
+          push_task(A, c, epoch);
+      } else if (ex[s] && small) {
+        push_small(A, make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, 1));
+      } else if (ex[s]) {
         // the records written to buffer 1 by every thread are ordered before
         // this thread by the barrier; push_task's release store publishes them
         push_task(A, make_task(gbegin + b, cn, id, s, X.depth + 1, s ? R : L, 1), epoch);
@@ -1783,7 +1824,7 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
   // every thread takes the kept child from the unions it read (no barrier:
   // the node thread's write and release fence overlap the next split's
   // binning, which reads only the kept child's records)
-  if (!kGlobal && (keep ? nr : nl) <= kMicro) return false;
+  if (!kGlobal && (keep ? nr : nl) <= lim) return false;
   X = sub_node(X.b + (keep ? nl : 0), keep ? nr : nl, id, keep, X.depth + 1, p ^ 1, keep ? R : L);
   return !kGlobal || X.n > kSubMax;
 }
@@ -1858,7 +1899,7 @@ __device__ void sub_tree(const BuildArgs& A, SubSmem& S, const Task& t, int epoc
     S.mnext = 0;
     if (n <= kMicro) S.ml[S.nm++] = micro_pack(0, n, t.parent, t.side, 0, 0);
   }
-  if (n > kMicro) {  // the chain of larger children, split by the whole CTA
+  if (n > kMicro) {  // (a task of k_small's size comes here only when a scene is one)  // the chain of larger children, split by the whole CTA
     SubNode X = task_node(t, 0);
     for (int it = 0; cta_split<false>(A, S, X, it, t.begin, t.depth, epoch, ws); ++it) {
     }
@@ -1928,6 +1969,237 @@ __device__ void sub_loop(const BuildArgs& A, SubSmem& S, int epoch) {
 // (CTA per item) and then join the others, which take the subtree queue
 // (CTA per subtree).  Both run at once, so subtrees proceed while the big
 // nodes of other branches are still being split.
+// Joins the box (lo, hi) to x where a == b, as predicated instructions: a
+// branch here would cost a reconvergence per record.
+__device__ __forceinline__ void binb_join_if(BinB& x, unsigned a, unsigned b, float4 lo, float4 hi) {
+  asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %7, %8;\n\t@p add.s32 %0, %0, 1;\n\t@p min.f32 %1, %1, %9;\n\t"
+      "@p min.f32 %2, %2, %10;\n\t@p min.f32 %3, %3, %11;\n\t@p max.f32 %4, %4, %12;\n\t"
+      "@p max.f32 %5, %5, %13;\n\t@p max.f32 %6, %6, %14;\n\t}"
+      : "+r"(x.n), "+f"(x.l0), "+f"(x.l1), "+f"(x.l2), "+f"(x.h0), "+f"(x.h1), "+f"(x.h2)
+      : "r"(a), "r"(b), "f"(lo.x), "f"(lo.y), "f"(lo.z), "f"(hi.x), "f"(hi.y), "f"(hi.z));
+}
+
+// Split a node of 33 .. kWarpMax records (src, shared memory) with one warp.
+// Lane s holds bin s: every lane reads every record (broadcasts) and joins
+// those of its own bin in registers, as many axes at a time as 32 lanes hold
+// (at most 16 bins in all: the half-warps take every other record each), so
+// there is nothing to clear, no atomic and no bin in memory.  The records
+// return to src in the order of the stable partition.  The same bins, costs
+// and order as cta_split's, so the same tree.  Returns the records on the
+// left; both children's boxes in L and R.
+__device__ __forceinline__ int warp_split(const BuildArgs& A, unsigned* idx, float4* src, int n, BinU& L, BinU& R) {
+  constexpr int kPer = kWarpMax / 32;
+  const int lane = threadIdx.x & 31;
+  const int K = A.K;
+  unsigned ext[6] = {0u, 0u, 0u, 0u, 0u, 0u};  // centre bounds: ~code of the least, code of the largest
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int k = r * 32 + lane;
+    if (k < n) {
+      const float4 lo = src[2 * k], hi = src[2 * k + 1];
+      const unsigned u0 = ucode(centre(lo.x, hi.x)), u1 = ucode(centre(lo.y, hi.y)), u2 = ucode(centre(lo.z, hi.z));
+      ext[0] = max(ext[0], ~u0);
+      ext[1] = max(ext[1], ~u1);
+      ext[2] = max(ext[2], ~u2);
+      ext[3] = max(ext[3], u0);
+      ext[4] = max(ext[4], u1);
+      ext[5] = max(ext[5], u2);
+    }
+  }
+  __syncwarp();
+  float cmin[3], scl[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    cmin[a] = uval(~__reduce_max_sync(kFull, ext[a]));
+    scl[a] = bin_scale(cmin[a], uval(__reduce_max_sync(kFull, ext[3 + a])), K);
+  }
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int k = r * 32 + lane;
+    if (k < n) {
+      const float4 lo = src[2 * k], hi = src[2 * k + 1];
+      idx[k] = (unsigned)bin_of(centre(lo.x, hi.x), cmin[0], scl[0], K) |
+               (unsigned)bin_of(centre(lo.y, hi.y), cmin[1], scl[1], K) << 8 |
+               (unsigned)bin_of(centre(lo.z, hi.z), cmin[2], scl[2], K) << 16;
+    }
+  }
+  __syncwarp();
+  Split best;
+  split_none(best);
+  for (int a0 = 0; a0 < 3;) {
+    const int m = min(3 - a0, 32 / K);
+    if (m >= 2 || __any_sync(kFull, sel3(scl[0], scl[1], scl[2], a0) > 0.f)) {
+      const bool half = m * K <= 16;
+      const int ll = half ? lane & 15 : lane;
+      const int g = ll / K, sl = ll - g * K;
+      bool in = g < m;
+      const int shift = 8 * (a0 + (in ? g : 0));
+      const unsigned want = in ? (unsigned)sl : 0xffffffffu;
+      const int step = half ? 2 : 1;
+      BinB x = binb_empty();
+#pragma unroll 4
+      for (int k = half ? lane >> 4 : 0; k < n; k += step) {
+        const unsigned w = idx[k];
+        const float4 lo = src[2 * k], hi = src[2 * k + 1];
+        binb_join_if(x, (w >> shift) & 255u, want, lo, hi);
+      }
+      __syncwarp();
+      if (half) {
+        x = binb_join(x, binb_xor(x, 16));
+        in = in && lane < 16;
+        if (!in) x = binb_empty();
+      }
+      eval_bins<false>(x, nullptr, in, in ? g : 32, sl, K, n, a0, A.cp, best);
+    }
+    a0 += m;
+  }
+  int axis = -1, plane = 0, nl = n / 2;
+  if (best.cand != INT_MAX) {
+    axis = best.cand / (K - 1);
+    plane = 1 + best.cand % (K - 1);
+    nl = best.L.n;
+  }
+  float4 lo[kPer], hi[kPer];
+  int dest[kPer];
+  int lrun = 0;
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    const int k = r * 32 + lane;
+    bool left = false;
+    if (k < n) {
+      lo[r] = src[2 * k];
+      hi[r] = src[2 * k + 1];
+      left = axis >= 0 ? (int)((idx[k] >> (8 * axis)) & 255u) < plane : k < nl;
+    }
+    __syncwarp();
+    const unsigned b = __ballot_sync(kFull, left);
+    const int before = lrun + __popc(b & ((1u << lane) - 1u));  // records on the left before k
+    dest[r] = left ? before : nl + k - before;
+    lrun += __popc(b);
+  }
+  if (lane == 0 && lrun != nl) set_status(A.ctl, kStBadSplit, 7);
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    if (r * 32 + lane < n && dest[r] < n) {
+      src[2 * dest[r]] = lo[r];
+      src[2 * dest[r] + 1] = hi[r];
+    }
+  }
+  L = best.L;
+  R = best.R;
+  if (__any_sync(kFull, axis < 0)) {  // no usable plane: the halves' boxes from their records
+    unsigned u[12];  // codes of the left's box (lo complemented), then the right's
+#pragma unroll
+    for (int q = 0; q < 12; ++q) u[q] = 0u;
+#pragma unroll
+    for (int r = 0; r < kPer; ++r) {
+      if (r * 32 + lane < n) {
+        const unsigned c[6] = {~ucode(lo[r].x), ~ucode(lo[r].y), ~ucode(lo[r].z),
+                               ucode(hi[r].x), ucode(hi[r].y), ucode(hi[r].z)};
+        const bool left = dest[r] < nl;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          u[q] = max(u[q], left ? c[q] : 0u);
+          u[6 + q] = max(u[6 + q], left ? 0u : c[q]);
+        }
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 12; ++q) u[q] = __reduce_max_sync(kFull, u[q]);
+    L.l0 = uval(~u[0]), L.l1 = uval(~u[1]), L.l2 = uval(~u[2]);
+    L.h0 = uval(u[3]), L.h1 = uval(u[4]), L.h2 = uval(u[5]);
+    R.l0 = uval(~u[6]), R.l1 = uval(~u[7]), R.l2 = uval(~u[8]);
+    R.h0 = uval(u[9]), R.h1 = uval(u[10]), R.h2 = uval(u[11]);
+  }
+  __syncwarp();  // src is written before any lane reads it again
+  return nl;
+}
+
+// The subtrees of a large scene's nodes of at most kWarpMax records, a warp
+// each from its node to its leaves: the records in shared memory, the larger
+// child kept, the other on the warp's stack.  A CTA split of so few records
+// waits at its barriers most of the time (7k cycles of 8 warps for 33-64
+// records); here every warp of the SM has a node of its own and the issue of
+// instructions bounds it (13.2M-triangle metro: 778k nodes of at most 32
+// records and 767k splits in 5.3 ms, 14.9 ms inside the split kernel).  24
+// warps per SM (80 registers).
+struct SmallSmem {
+  float4 rec[kWarps][2 * kWarpMax];
+  unsigned idx[kWarps][kWarpMax];
+  int4 stack[kWarps][kWarpMax / 2];  // (first record, records | side << 16, parent, depth): disjoint, >= 2 records
+};
+
+__global__ void __launch_bounds__(kBlock, 3) k_small(BuildArgs A) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ SmallSmem S;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int epoch = __ldcg(&A.ctl->epoch);
+  const int count = __shfl_sync(kFull, __ldcg(&A.ctl->sq_count), 0);
+  float4* rec = S.rec[warp];
+  int4* stack = S.stack[warp];
+  WarpStats ws{0, 0, 0, 0};
+  for (;;) {
+    int i = 0;
+    if (lane == 0) i = atomicAdd(&A.ctl->sq_head, 1);
+    i = __shfl_sync(kFull, i, 0);
+    if (i >= count) break;
+    const int4* q = reinterpret_cast<const int4*>(A.qa + (A.qa_cap - 1 - i));
+    const int4 t0 = __ldcg(q), t1 = __ldcg(q + 1), t2 = __ldcg(q + 2);
+    const int begin = t0.x;
+    int n = __shfl_sync(kFull, t0.y, 0), b = 0, parent = t0.z, side = t0.w, depth = t1.w, sp = 0;
+    if (begin < 0 || n < 2 || n > kWarpMax || begin > A.n - n) {
+      if (lane == 0) set_status(A.ctl, kStBadSplit, 8);
+      continue;
+    }
+    const float4* g = A.rec[t2.w & 1] + 2 * (size_t)begin;
+    for (int k = lane; k < 2 * n; k += 32) rec[k] = __ldcg(g + k);
+    __syncwarp();
+    for (;;) {
+      while (n > kMicro) {
+        float4* src = rec + 2 * b;
+        BinU L, R;
+        const int nl = __shfl_sync(kFull, warp_split(A, S.idx[warp], src, n, L, R), 0), nr = n - nl;
+        const bool leafl = nl <= A.max_leaf, leafr = nr <= A.max_leaf;
+        const int id = begin + b + nl - 1;
+        const int keep = nl >= nr ? 0 : 1;
+        if (leafl) leaf_out<false>(A, src, begin + b, nl, lane, 32);
+        if (leafr) leaf_out<false>(A, src + 2 * nl, begin + b + nl, nr, lane, 32);
+        if (lane == 0) {
+          write_node(A, id, parent, side, L, leafl ? leaf_ref(begin + b, nl) : INT_MAX, nl, R,
+                     leafr ? leaf_ref(begin + b + nl, nr) : INT_MAX, nr, epoch);
+          note_node(ws, nl, nr, leafl, leafr, depth);
+          if (!(keep ? leafl : leafr))  // the smaller child
+            stack[sp] = keep ? make_int4(b, nl, id, depth + 1) : make_int4(b + nl, nr | (1 << 16), id, depth + 1);
+        }
+        __syncwarp();
+        sp += (keep ? leafl : leafr) ? 0 : 1;
+        parent = id;
+        side = keep;
+        ++depth;
+        b += keep ? nl : 0;
+        n = keep ? nr : nl;
+      }
+      if (n > A.max_leaf) micro_sort_build(A, rec + 2 * b, begin + b, n, parent, side, depth, epoch, ws);
+      if (sp == 0) break;
+      const int4 e = stack[--sp];
+      b = e.x;
+      n = __shfl_sync(kFull, e.y & 0xffff, 0);
+      side = e.y >> 16;
+      parent = e.z;
+      depth = e.w;
+    }
+    __syncwarp();
+  }
+  if (lane == 0) {
+    if (ws.n_int) atomicAdd(&A.ctl->n_internal, ws.n_int);
+    if (ws.n_leaf) atomicAdd(&A.ctl->n_leaves, ws.n_leaf);
+    if (ws.big) atomicMax(&A.ctl->max_leaf_size, ws.big);
+    if (ws.deep) atomicMax(&A.ctl->depth2, ws.deep);
+  }
+}
+
 union SplitSmem {
   TopSmem top;
   SubSmem sub;
@@ -2311,6 +2583,13 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   A.n_all = (int)s->n_tri;
   A.K = p.bins;
   A.max_leaf = p.max_leaf;
+  // k_small pays where the subtrees fill the device and the split kernel is
+  // bound by what they cost, not by the longest of them.  Builds without it,
+  // with 64 and with 128 records a node, alpha 1: 60k triangles 0.241 /
+  // 0.255 / 0.289 ms, 279k 0.647 / 0.557 / 0.548, 600k 1.36 / 1.14 / 1.09, 4M
+  // 7.70 / 5.93 / 5.33; alpha 0.7: 199k 0.716 / 0.737 / 0.750, 279k 0.912 /
+  // 0.838 / 0.871, 600k 1.81 / 1.67 / 1.63, 4M 11.4 / 9.46 / 8.70.
+  A.wsm = n < 240000 ? 0 : (n < 500000 ? kWarpMax / 2 : kWarpMax);
   A.big = g.big;
   A.chunk = g.chunk;
   A.rpt = g.rpt;
@@ -2351,6 +2630,10 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   if (s->split_ev[0] && (e = cudaEventRecordWithFlags(s->split_ev[0], st, evflags))) return e;
   if ((e = launch(k_split, split_per_sm * nsm, sizeof(SplitSmem), st, true, A))) return e;
   if (s->split_ev[1] && (e = cudaEventRecordWithFlags(s->split_ev[1], st, evflags))) return e;
+  if (A.wsm) {
+    if ((e = launch(k_small, 3 * nsm, 0, st, true, A))) return e;
+    count_launches(1);
+  }
   if ((e = launch(k_post, gp, 0, st, true, A))) return e;
   count_launches(4);
   return cudaSuccess;

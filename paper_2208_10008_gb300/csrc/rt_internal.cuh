@@ -174,8 +174,8 @@ struct BuildCtl {
   // subtree task queue (CTA per task)
   int qa_head, qa_tail, qa_pending, pad3;
   int pad_a[20];
-  // pools of one build: top task slots, count slots
-  int t_slot_next, t_cnt_next, pad1, pad2;
+  // pools of one build: top task slots, count slots; k_small's nodes, those taken
+  int t_slot_next, t_cnt_next, sq_count, sq_head;
   int pad_b[28];
   // tree facts
   int n_internal, n_leaves, depth2, max_leaf_size;
