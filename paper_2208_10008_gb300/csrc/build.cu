@@ -44,6 +44,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <climits>
+#include <type_traits>
 
 #include "rt_internal.cuh"
 
@@ -55,7 +56,10 @@ constexpr int kWarps = kBlock / 32;
 constexpr int kBinVals = 13;  // count, box lo xyz, box hi xyz, centre lo xyz, centre hi xyz
 constexpr int kBinWords = 3 * kMaxBins * kBinVals;
 constexpr int kCntStride = 3 * kMaxBins;
-constexpr int kMaxRpt = 4;     // records per thread of a big node's chunk
+constexpr int kMaxRpt = 8;     // records per thread of a big node's chunk
+constexpr int kRegRpt = 4;     // at most, where they stay in registers
+constexpr int kStage = 2048;   // of a chunk's records in shared memory at a time
+constexpr int kLargeScene = 240000;  // records from which a build is bound by work and not by its longest chain
 constexpr int kBigMin = 1024;  // big nodes have more triangles than this
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -226,6 +230,49 @@ __device__ __forceinline__ void bin_add_runs(int cell, const int* e, unsigned* b
       if (cnt) atomicAdd(cnt + e[a], m);
     }
   }
+}
+
+// A lane's run of records of one cell: the code maxima, the count, and per
+// axis the word offset of its bin (from the bins) and of its count (<< 16,
+// from the counts).
+struct CellRun {
+  unsigned v[12], n, off[3];
+  int cell;  // -1: none
+};
+
+__device__ __forceinline__ void run_add(const CellRun& r, unsigned* bins, unsigned* cnt) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    unsigned* b = bins + (r.off[a] & 0xffffu);
+    atomicAdd(b, r.n);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) atomicMax(b + 1 + q, r.v[q]);
+    atomicAdd(cnt + (r.off[a] >> 16), r.n);
+  }
+}
+
+// Add the run that every lane holds, joined first with the adjacent lanes'
+// runs of the same cell by a segmented warp scan (as many steps as the
+// longest stretch of equal cells needs); the last lane of a stretch issues
+// the atomics.  All 32 lanes of the warp must call.
+__device__ __forceinline__ void run_add_warp(CellRun r, unsigned* bins, unsigned* cnt) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  const int prev = __shfl_up_sync(kFull, r.cell, 1), next = __shfl_down_sync(kFull, r.cell, 1);
+  const bool head = lane == 0 || prev != r.cell, tail = lane == 31 || next != r.cell;
+  const unsigned heads = __ballot_sync(kFull, head);
+  const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));  // first lane of the stretch
+  const int span = (int)__reduce_max_sync(kFull, (unsigned)(lane - start));
+#pragma unroll 1
+  for (int o = 1; o <= span; o <<= 1) {
+    const int from = max(lane - o, start);
+    const unsigned m = __shfl_sync(kFull, r.n, from);
+    r.n += lane - o >= start ? m : 0u;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) r.v[q] = max(r.v[q], __shfl_sync(kFull, r.v[q], from));  // (idempotent)
+  }
+  if (tail && r.cell >= 0) run_add(r, bins, cnt);
+  __syncwarp();
 }
 
 // ------------------------------------------------------------------ Eq. 2 evaluation
@@ -795,6 +842,11 @@ __device__ __forceinline__ void note_node(WarpStats& ws, int nl, int nr, bool le
 }
 
 // ------------------------------------------------------------------ big nodes
+// Shared-memory place of record k of a stage, in float4: four records and
+// 16 bytes of padding per thread, so that 16-byte reads of consecutive
+// records by consecutive lanes fall on distinct banks.
+__device__ __forceinline__ int stage_at(int k) { return (k >> 2) * 9 + (k & 3) * 2; }
+
 struct TopSmem {
   unsigned pbins[kBinWords];
   unsigned cbins[2][kBinWords];
@@ -808,6 +860,13 @@ struct TopSmem {
   int4 plan[2];
   Task ptask[2];  // subtree-sized children the emit hands to the subtree queue
   int np;
+};
+
+// With a stage of the chunk's records.
+struct StagedSmem {
+  TopSmem top;
+  alignas(16) float4 rec[kStage / 4 * 9];  // (stage_at)
+  unsigned short order[kStage];            // its records, the left ones first
 };
 
 __device__ __forceinline__ int block_sum(int v, int* red) {
@@ -856,35 +915,36 @@ __device__ void top_emit(const BuildArgs& A, TopSmem& S, const TopTask& T, int s
                          const BinU& cu0, const BinU& cu1, bool top0, bool top1, int nch0, int nch1, int cfirst0,
                          int cfirst1, WarpStats& ts);
 
-// Chunk 0 of a big node, as soon as its split is known: reserve what the
-// node's big children will need (two task slots and the count slots for
-// their own children, their chunk items) and clear what their chunks will
-// fill, so that the CTA finishing the node's last chunk only writes and
-// publishes.  The clearing is ordered before that CTA's emit by chunk 0's
-// release of its done count.
-__device__ void top_plan(const BuildArgs& A, TopSmem& S, int slot, bool top0, bool top1, int nch0, int nch1) {
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    int cs[2] = {-1, -1}, cr[2] = {-1, -1}, ib[2] = {-1, -1};
-    // every reservation is issued before any result is used: one round trip
+// Chunk 0 of a big node, as soon as its split is known: one thread reserves
+// what the node's big children will need (two task slots and the count slots
+// for their own children, their chunk items) while the chunk is partitioned;
+// then the CTA clears what their chunks will fill, so that the CTA finishing
+// the node's last chunk only writes and publishes.  The clearing is ordered
+// before that CTA's emit by chunk 0's release of its done count.
+__device__ __forceinline__ void top_reserve(const BuildArgs& A, TopSmem& S, int slot, bool top0, bool top1, int nch0,
+                                            int nch1) {
+  int cs[2] = {-1, -1}, cr[2] = {-1, -1}, ib[2] = {-1, -1};
+  // every reservation is issued before any result is used: one round trip
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      if (!(s ? top1 : top0)) continue;
-      const int ncs = s ? nch1 : nch0;
-      cs[s] = reserve(&A.ctl->t_slot_next, 2, A.cap_t);
-      cr[s] = reserve(&A.ctl->t_cnt_next, ncs + 2, A.cap_c);
-      ib[s] = reserve(&A.ctl->ti_tail, ncs, A.cap_c);
-    }
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int ncs = s ? nch1 : nch0;
-      const int4 pl = (cs[s] >= 0 && cr[s] >= 0 && ib[s] >= 0) ? make_int4(cs[s], cr[s], ib[s], ncs + 2)
-                                                             : make_int4(-1, -1, -1, 0);
-      S.plan[s] = pl;
-      A.tplan[2 * slot + s] = pl;
-    }
+  for (int s = 0; s < 2; ++s) {
+    if (!(s ? top1 : top0)) continue;
+    const int ncs = s ? nch1 : nch0;
+    cs[s] = reserve(&A.ctl->t_slot_next, 2, A.cap_t);
+    cr[s] = reserve(&A.ctl->t_cnt_next, ncs + 2, A.cap_c);
+    ib[s] = reserve(&A.ctl->ti_tail, ncs, A.cap_c);
   }
-  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int ncs = s ? nch1 : nch0;
+    const int4 pl =
+        (cs[s] >= 0 && cr[s] >= 0 && ib[s] >= 0) ? make_int4(cs[s], cr[s], ib[s], ncs + 2) : make_int4(-1, -1, -1, 0);
+    S.plan[s] = pl;
+    A.tplan[2 * slot + s] = pl;
+  }
+}
+// (after a barrier: the partition's)
+__device__ __forceinline__ void top_clear(const BuildArgs& A, TopSmem& S) {
+  const int tid = threadIdx.x;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const int4 pl = S.plan[s];
@@ -908,8 +968,10 @@ __device__ void top_plan(const BuildArgs& A, TopSmem& S, int slot, bool top0, bo
 // that finishes the node's last chunk writes the node and creates its
 // children: big ones get their chunk items, the others go to the subtree
 // queue.  No CTA ever waits for another.
+template <bool kStaged>
 __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int slot, int j, int epoch,
                           WarpStats& ts) {
+  StagedSmem& G = reinterpret_cast<StagedSmem&>(S);  // (where kStaged)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = A.K, K3 = 3 * K, CH = A.chunk;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -919,16 +981,32 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   float4* dst = A.rec[par ^ 1];
   const int r0 = j * CH;
   const int rn = min(CH, n - r0);
-  // the chunk's records, in flight while the split is chosen
-  float4 lo[kMaxRpt], hi[kMaxRpt];
+  // the chunk's records go to shared memory stage by stage, the first while
+  // the split is chosen
+  auto fetch = [&](int g) {
+    const int m = min(kStage, rn - g * kStage);
+    if (m > 0) {
+      const float4* p = src + 2 * ((size_t)T.begin + r0 + g * kStage);
+      const unsigned to = (unsigned)__cvta_generic_to_shared(&G.rec[0]);
+      for (int i = tid; i < 2 * m; i += kBlock)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * (stage_at(i >> 1) + (i & 1))),
+                     "l"(p + i)
+                     : "memory");
+    }
+  };
+  float4 lo[kRegRpt], hi[kRegRpt];
+  if (kStaged) {
+    fetch(0);
+  } else {
 #pragma unroll
-  for (int r = 0; r < kMaxRpt; ++r) {
-    const int k = r * kBlock + tid;
-    lo[r] = hi[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < A.rpt && k < rn) {
-      const float4* p = src + 2 * ((size_t)T.begin + r0 + k);
-      lo[r] = __ldcg(p);
-      hi[r] = __ldcg(p + 1);
+    for (int r = 0; r < kRegRpt; ++r) {
+      const int k = r * kBlock + tid;
+      lo[r] = hi[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < A.rpt && k < rn) {
+        const float4* p = src + 2 * ((size_t)T.begin + r0 + k);
+        lo[r] = __ldcg(p);
+        hi[r] = __ldcg(p + 1);
+      }
     }
   }
   {
@@ -997,7 +1075,13 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   const bool top0 = nl > A.big, top1 = nr > A.big;
   const int nch0 = (nl + CH - 1) / CH, nch1 = (nr + CH - 1) / CH;
   const int cfirst0 = T.chunk_res, cfirst1 = T.chunk_res + nch0;
-  if (j == 0) top_plan(A, S, slot, top0, top1, nch0, nch1);
+  // (in a small scene the clearing too comes first: a level waits for its
+  // chunk 0, and the other chunks are few)
+  if (j == 0 && tid == kBlock - 1) top_reserve(A, S, slot, top0, top1, nch0, nch1);
+  if (!kStaged && j == 0) {
+    __syncthreads();
+    top_clear(A, S);
+  }
   const float cmin0[3] = {cu0.a0, cu0.a1, cu0.a2}, cmin1[3] = {cu1.a0, cu1.a1, cu1.a2};
   const float scl0[3] = {bin_scale(cu0.a0, cu0.b0, K), bin_scale(cu0.a1, cu0.b1, K), bin_scale(cu0.a2, cu0.b2, K)};
   const float scl1[3] = {bin_scale(cu1.a0, cu1.b0, K), bin_scale(cu1.a1, cu1.b1, K), bin_scale(cu1.a2, cu1.b2, K)};
@@ -1023,11 +1107,115 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   }
   const int rbase = r0 - lbase;
   const int dfirst0 = lbase / CH, dfirst1 = rbase / CH;
-  // stable partition of the chunk; the records of children that are big
-  // nodes too are binned for them on the way
+  const int dnext0 = (dfirst0 + 1) * CH, dnext1 = (dfirst1 + 1) * CH;  // first positions of the next child chunks
+  const float pcmin = sel3(cmin[0], cmin[1], cmin[2], axis < 0 ? 0 : axis);
+  const float pscl = sel3(scl[0], scl[1], scl[2], axis < 0 ? 0 : axis);
+  // stable partition of the chunk, a stage at a time; the records of children
+  // that are big nodes too are binned for them on the way.  A thread takes up
+  // to 8 consecutive records: runs of one cell (the records of a building, a
+  // wall) mostly lie within a thread or its neighbours, so that one scan of 12
+  // words by shuffles, which bound this step, serves 256 records and not 32.
   int lrun = 0, rrun = 0;
+  for (int g = 0; kStaged && g * kStage < rn; ++g) {
+    const int m = min(kStage, rn - g * kStage);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const float4* rec = G.rec;
+    const int c = (m + kBlock - 1) / kBlock, k0 = min(tid * c, m), k1 = min(k0 + c, m);
+    unsigned fl = 0;  // bit i: record k0 + i goes left
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      bool left;
+      if (axis >= 0) {
+        const float* q = reinterpret_cast<const float*>(rec + stage_at(k)) + axis;
+        left = bin_of(centre(q[0], q[4]), pcmin, pscl, K) < plane;
+      } else {
+        left = r0 + g * kStage + k < nl;
+      }
+      fl |= (unsigned)left << (k - k0);
+    }
+    __syncwarp();
+    int before = 0, wtot = 0;
 #pragma unroll
-  for (int r = 0; r < kMaxRpt; ++r) {
+    for (int r = 0; r < kStage / kBlock; ++r) {
+      const unsigned bal = __ballot_sync(kFull, (fl >> r) & 1u);
+      before += __popc(bal & lt_mask);
+      wtot += __popc(bal);
+    }
+    if (lane == 0) S.wl[warp] = wtot;
+    __syncthreads();
+    int tl = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const int v = S.wl[w];
+      before += w < warp ? v : 0;
+      tl += v;
+    }
+    int lp = before, rp = k0 - before;  // positions of the thread's next left and right record in the stage
+    CellRun run;
+    run.cell = -1;
+    run.n = 0;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) run.v[q] = 0u;
+    run.off[0] = run.off[1] = run.off[2] = 0u;
+    for (int r = 0; r < c; ++r) {  // (uniform)
+      const int k = k0 + r;
+      const bool valid = k < k1;
+      const bool left = (fl >> r) & 1u;
+      const int pos = left ? lp : rp;
+      if (valid) G.order[left ? pos : tl + pos] = (unsigned short)k;
+      lp += valid && left ? 1 : 0;
+      rp += valid && !left ? 1 : 0;
+      if (top0 || top1) {
+        const bool act = valid && (left ? top0 : top1);
+        const int kk = valid ? k : 0;
+        const float4 lo = rec[stage_at(kk)], hi = rec[stage_at(kk) + 1];
+        const float cx = centre(lo.x, hi.x), cy = centre(lo.y, hi.y), cz = centre(lo.z, hi.z);
+        const RecCodes rc = rec_codes(lo, hi, cx, cy, cz);
+        const int jj = left ? (lbase + lrun + pos >= dnext0 ? 1 : 0) : (rbase + rrun + pos >= dnext1 ? 1 : 0);
+        int cell = (left ? 0 : 2) + jj;
+        const unsigned cb = (unsigned)cell * kCntStride, bb = left ? 0u : (unsigned)kBinWords;
+        unsigned off[3];
+        const float cc[3] = {cx, cy, cz};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int b = bin_of(cc[a], left ? cmin0[a] : cmin1[a], left ? scl0[a] : scl1[a], K);
+          off[a] = (bb + (unsigned)((a * K + b) * kBinVals)) | (cb + (unsigned)(a * K + b)) << 16;
+          cell = cell * kMaxBins + b;
+        }
+        const bool fresh = act && cell != run.cell, out = fresh && run.cell >= 0;
+        if (__any_sync(kFull, out)) {
+          if (out) run_add(run, &S.cbins[0][0], &S.ccnt[0][0][0]);
+          __syncwarp();
+        }
+        run.n = fresh ? 1u : run.n + (act ? 1u : 0u);
+        run.cell = fresh ? cell : run.cell;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) run.off[a] = fresh ? off[a] : run.off[a];
+#pragma unroll
+        for (int q = 0; q < 12; ++q) run.v[q] = fresh ? rc.v[q] : max(run.v[q], act ? rc.v[q] : 0u);
+      }
+    }
+    if (top0 || top1) run_add_warp(run, &S.cbins[0][0], &S.ccnt[0][0][0]);
+    __syncthreads();
+    // the records leave in the order of their places, 512 bytes a warp
+    for (int i = tid; i < 2 * m; i += kBlock) {
+      const int p = i >> 1;
+      const bool left = p < tl;
+      const int dest = left ? lbase + lrun + p : rbase + rrun + p - tl;
+      const float4 v = rec[stage_at(G.order[p]) + (i & 1)];
+      if (dest < (left ? nl : nr))
+        dst[2 * ((size_t)T.begin + (left ? 0 : nl) + dest) + (i & 1)] = v;
+      else
+        set_status(A.ctl, kStBadSplit, 3);
+    }
+    lrun += tl;
+    rrun += m - tl;
+    __syncthreads();  // the stage is free
+    fetch(g + 1);
+  }
+#pragma unroll
+  for (int r = 0; !kStaged && r < kRegRpt; ++r) {  // a round of 256 records, a record a thread
     if (r >= A.rpt || r * kBlock >= rn) break;
     const int k = r * kBlock + tid;
     const bool valid = k < rn;
@@ -1066,23 +1254,24 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
     }
     if (top0 || top1) {
       const bool act = valid && (s ? top1 : top0);
-      const int jj = dest / CH - (s ? dfirst1 : dfirst0);
+      const int jj = (dest / CH - (s ? dfirst1 : dfirst0)) & 1;
       const float cx = centre(lo[r].x, hi[r].x), cy = centre(lo[r].y, hi[r].y), cz = centre(lo[r].z, hi[r].z);
       const float cc[3] = {cx, cy, cz};
       const RecCodes rc = rec_codes(lo[r], hi[r], cx, cy, cz);
-      int e[3], cell = s * 2 + (jj & 1);
+      int e[3], cell = s * 2 + jj;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const int b = s ? bin_of(cc[a], cmin1[a], scl1[a], K) : bin_of(cc[a], cmin0[a], scl0[a], K);
         e[a] = a * K + b;
         cell = cell * kMaxBins + b;
       }
-      bin_add_runs(act ? cell : -1, e, &S.cbins[s][0], &S.ccnt[s][jj & 1][0], rc);
+      bin_add_runs(act ? cell : -1, e, &S.cbins[s][0], &S.ccnt[s][jj][0], rc);
     }
     lrun += rtot;
     rrun += min(kBlock, rn - r * kBlock) - rtot;
     __syncthreads();
   }
+  if (kStaged && j == 0) top_clear(A, S);
   // the children's bins and chunk counts
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
@@ -1200,6 +1389,7 @@ __device__ void top_emit(const BuildArgs& A, TopSmem& S, const TopTask& T, int s
 }
 
 // Chunk j of big node `slot`, after checking the node's fields.
+template <bool kStaged>
 __device__ void top_item(const BuildArgs& A, TopSmem& S, int slot, int j, int epoch, WarpStats& ts) {
   const int tid = threadIdx.x;
   TopTask T;
@@ -1225,10 +1415,11 @@ __device__ void top_item(const BuildArgs& A, TopSmem& S, int slot, int j, int ep
   if (!ok) {
     if (tid == 0) set_status(A.ctl, kStBadSplit, 4);
   } else {
-    top_chunk(A, S, T, slot, j, epoch, ts);
+    top_chunk<kStaged>(A, S, T, slot, j, epoch, ts);
   }
 }
 
+template <bool kStaged>
 __device__ void top_loop(const BuildArgs& A, TopSmem& S, int epoch) {
   WarpStats ts{0, 0, 0, 0};  // thread 0's tally of the nodes this CTA wrote
   for (;;) {
@@ -1237,7 +1428,7 @@ __device__ void top_loop(const BuildArgs& A, TopSmem& S, int epoch) {
     const int2 it = S.item;
     __syncthreads();
     if (it.x < 0) break;
-    top_item(A, S, it.x, it.y, epoch, ts);
+    top_item<kStaged>(A, S, it.x, it.y, epoch, ts);
     __syncthreads();
     // release: the subtree tasks this item pushed are counted before the
     // item stops counting (the warps' exit test reads ti_pending first)
@@ -2200,19 +2391,28 @@ __global__ void __launch_bounds__(kBlock, 3) k_small(BuildArgs A) {
   }
 }
 
+template <bool kStaged>
 union SplitSmem {
-  TopSmem top;
+  std::conditional_t<kStaged, StagedSmem, TopSmem> top;
   SubSmem sub;
 };
 
+// kStaged (large scenes): the big nodes' chunks go through shared memory, up
+// to 8 consecutive records a thread, instead of registers, a record a thread
+// and round.  The shuffles of the children's binning bound a chunk, 60 for 32
+// records (an SM does one every two cycles); staged, 65 serve 256.  Builds of
+// 600k triangles 1.09 -> 0.81 ms at alpha 1 and 1.63 -> 1.39 at 0.7, 4M 5.35 ->
+// 4.55 and 8.71 -> 7.46; but 20k 0.203 -> 0.210, 199k 0.717 -> 0.765 at 0.7,
+// where a level's latency counts and a chunk has few records.
+template <bool kStaged>
 __global__ void __launch_bounds__(kBlock, 2) k_split(BuildArgs A) {
   pdl_wait();
   pdl_launch();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SplitSmem& S = *reinterpret_cast<SplitSmem*>(smem_raw);
+  SplitSmem<kStaged>& S = *reinterpret_cast<SplitSmem<kStaged>*>(smem_raw);
   const int epoch = __ldcg(&A.ctl->epoch);
   if ((int)blockIdx.x < A.top_ctas) {
-    top_loop(A, S.top, epoch);
+    top_loop<kStaged>(A, reinterpret_cast<TopSmem&>(S), epoch);
     __syncthreads();
   }
   sub_loop(A, S.sub, epoch);
@@ -2475,6 +2675,8 @@ __global__ void __launch_bounds__(kBlock) k_post(BuildArgs A) {
   }
 }
 
+size_t split_smem(bool staged) { return staged ? sizeof(SplitSmem<true>) : sizeof(SplitSmem<false>); }
+
 int sm_count() {
   static int n = 0;
   if (!n) {
@@ -2510,7 +2712,10 @@ BuildGeom build_geometry(int64_t n, int nsm) {
   const int64_t T = n < 1 ? 1 : n;
   g.big = (int)std::max<int64_t>(kBigMin, (T + 4095) / 4096);
   int64_t rpt = (T + (int64_t)nsm * 512 - 1) / ((int64_t)nsm * 512);
-  rpt = std::min<int64_t>(std::max<int64_t>(rpt, 1), kMaxRpt);
+  // (8 from a million records: 1.2M 1.53 -> 1.37 ms at alpha 1, 2.52 -> 2.44 at
+  // 0.7, 13.2M 30.8 -> 27.1; 400k 0.640 -> 0.660 and 1.05 -> 1.10; 16 gains
+  // nothing more)
+  rpt = std::min<int64_t>(std::max<int64_t>(rpt, 1), T >= 1000000 ? kMaxRpt : kRegRpt);
   g.rpt = (int)rpt;
   g.chunk = kBlock * g.rpt;
   // Pools of one build (a full pool sends further big nodes to the subtree queue,
@@ -2589,7 +2794,8 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   // 0.255 / 0.289 ms, 279k 0.647 / 0.557 / 0.548, 600k 1.36 / 1.14 / 1.09, 4M
   // 7.70 / 5.93 / 5.33; alpha 0.7: 199k 0.716 / 0.737 / 0.750, 279k 0.912 /
   // 0.838 / 0.871, 600k 1.81 / 1.67 / 1.63, 4M 11.4 / 9.46 / 8.70.
-  A.wsm = n < 240000 ? 0 : (n < 500000 ? kWarpMax / 2 : kWarpMax);
+  const bool large = n >= kLargeScene;
+  A.wsm = !large ? 0 : (n < 500000 ? kWarpMax / 2 : kWarpMax);
   A.big = g.big;
   A.chunk = g.chunk;
   A.rpt = g.rpt;
@@ -2599,19 +2805,23 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   static bool attr = false;
   static int split_per_sm = 2;  // resident split CTAs per SM (at most 2)
   if (!attr) {
-    if ((e = cudaFuncSetAttribute(k_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SplitSmem))))
-      return e;
-    int occ = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_split, kBlock, sizeof(SplitSmem)))) return e;
+    int occ = 2;
+    for (bool staged : {false, true}) {
+      void (*k)(BuildArgs) = staged ? k_split<true> : k_split<false>;
+      const size_t sm = split_smem(staged);
+      if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm))) return e;
+      int o = 0;
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, kBlock, sm))) return e;
+      occ = std::min(occ, o);
+    }
     split_per_sm = std::max(1, std::min(2, occ));
     attr = true;
   }
   // the big-node chunks go to the first nsm CTAs, which then join the rest on
   // the subtree queue, so that subtrees proceed while other branches' big
-  // nodes are split; when a depth has many more chunks than SMs (large
-  // scenes) every CTA takes chunks first
-  const int64_t nchunks = (n + g.chunk - 1) / g.chunk;
-  A.top_ctas = n > g.big ? (nchunks > 8 * (int64_t)nsm ? split_per_sm * nsm : nsm) : 0;
+  // nodes are split; in large scenes every CTA takes chunks first (475k
+  // triangles 1.55 -> 1.50 ms)
+  A.top_ctas = n > g.big ? (large ? split_per_sm * nsm : nsm) : 0;
   const DebugHooks dh = debug_hooks();
   A.spin_limit = dh.spin_limit > 0 ? dh.spin_limit : kSpinLimit;
   A.phantom_tasks = dh.phantom_tasks;
@@ -2628,7 +2838,8 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   if (s->split_ev[0] && (e = cudaStreamIsCapturing(st, &cs))) return e;
   const unsigned evflags = cs == cudaStreamCaptureStatusNone ? cudaEventRecordDefault : cudaEventRecordExternal;
   if (s->split_ev[0] && (e = cudaEventRecordWithFlags(s->split_ev[0], st, evflags))) return e;
-  if ((e = launch(k_split, split_per_sm * nsm, sizeof(SplitSmem), st, true, A))) return e;
+  if ((e = launch(large ? k_split<true> : k_split<false>, split_per_sm * nsm, split_smem(large), st, true, A)))
+    return e;
   if (s->split_ev[1] && (e = cudaEventRecordWithFlags(s->split_ev[1], st, evflags))) return e;
   if (A.wsm) {
     if ((e = launch(k_small, 3 * nsm, 0, st, true, A))) return e;

@@ -67,13 +67,13 @@ def _city(n, seed=4):
     return np.concatenate([city + np.float32([3100.0 * (i % side), 3100.0 * (i // side), 0.0]) for i in range(k)])
 
 
-def _check_nodes(orc, tris, ex, alpha, src, bins, pick):
-    """Every node x with pick(records of x) true (at most 1500, seeded) is split at an Eq. 2 minimum."""
+def _check_nodes(orc, tris, ex, alpha, src, bins, pick, most=1500):
+    """Every node x with pick(records of x) true (at most `most`, seeded) is split at an Eq. 2 minimum."""
     first, cnt, nl = E.node_ranges(ex)
     assert np.array_equal(np.sort(ex["prims"]), np.arange(len(tris)))
     chk = E.Checker(orc, tris, alpha, src, dist_norm=1, bins=bins)
     nodes = np.nonzero(pick(cnt))[0]
-    nodes = np.random.default_rng(0).permutation(nodes)[:1500]
+    nodes = np.random.default_rng(0).permutation(nodes)[:most]
     keys = E.morton_keys(chk.lo, chk.hi)
     for x in nodes:
         ids = ex["prims"][first[x]: first[x] + cnt[x]]
@@ -105,6 +105,17 @@ def test_small_nodes_of_large_scenes(rb, orc, n, bins, max_leaf, alpha):
     rb.rt_bvh_build(s, source=src, alpha=alpha, max_leaf=max_leaf, bins=bins, dist_norm=1)
     again = rb.rt_bvh_export(s)
     assert all(np.array_equal(ex[k], again[k]) for k in ("child", "leaf_first", "leaf_count", "prims"))
+
+
+@pytest.mark.parametrize("n,bins", [(240000, 16), (300001, 32), (999999, 8), (1000003, 16)])
+@pytest.mark.parametrize("alpha", [1.0, 0.7])
+def test_big_nodes_of_large_scenes(rb, orc, n, bins, alpha):
+    """Chunks of 1024 and 2048 records through shared memory, ragged last ones among them."""
+    tris = _city(n)[:n]
+    src = (1500.0, 1500.0, 25.0)
+    _, ex = _build(rb, tris, src, alpha=alpha, max_leaf=4, bins=bins, dist_norm=1)
+    assert _check_nodes(orc, tris, ex, alpha, src, bins, lambda c: (c > 1024) & (c < 20000), 60) == 60
+    assert _check_nodes(orc, tris, ex, alpha, src, bins, lambda c: c >= 60000, 3) == 3
 
 
 def test_centroids_without_extent_in_a_large_scene(rb, orc):
