@@ -95,7 +95,7 @@ def alu_roofline(nodes_per_ray, tris_per_ray, rays, ms, n_sm, sm_mhz, width=4):
     achieved = ops_per_ray * rays / (ms * 1e-3) / 1e12
     peak = n_sm * 128 * sm_mhz * 1e6 / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
-            "ops_per_ray": ops_per_ray, "kernel": "k_trace + k_retest64 (one rt_trace_closest)",
+            "ops_per_ray": ops_per_ray, "kernel": "k_trace (one rt_trace_closest)",
             "peak_source": "%d SMs x 128 FP32 lanes x %.0f MHz (median SM clock under load)" % (n_sm, sm_mhz),
             "note": "estimated operation counts; the walk issues integer, load and stack instructions besides "
                     "these, so the issue rate (profiled) is higher than this fraction"}
@@ -372,7 +372,7 @@ def run_large(rtbvh, torch, hbm, runs=3):
                          "peak": hbm, "unit": "GB/s",
                          "frac": traffic / (ms_trace * 1e-3) / 1e9 / hbm if traffic else None,
                          "traffic": traffic, "traffic_unit": "bytes per launch",
-                         "traffic_source": ncu_src, "kernel": "k_trace + k_retest64",
+                         "traffic_source": ncu_src, "kernel": "k_trace",
                          "algorithmic_bytes_per_ray": per_ray, "algorithmic_gbs": gbs,
                          "note": "achieved = DRAM bytes of the launch (ncu) over its event time: the fraction of "
                                  "HBM the walk really uses.  The algorithmic bytes count every node and triangle "
@@ -626,7 +626,7 @@ NCU_TRAFFIC = {
     "k_split": (1.747968e6 + 768.0, "ncu capture of k_split in the timed steps, medium city, autotuned tree "
                                     "(profiles/k_split_medium_city.md)"),
     "k_trace": (21.461504e6 + 17920.0, "ncu capture of k_trace<0,0,128,64,0,4> in the timed steps, medium "
-                                       "city (k_retest64 not included; profiles/k_trace_medium_city.md)"),
+                                       "city (profiles/k_trace_medium_city.md)"),
 }
 
 
@@ -852,7 +852,7 @@ def run_ours(args):
                                  "with L2-only loads",
                   "traffic": NCU_TRAFFIC["k_trace"][0], "traffic_unit": "bytes per launch",
                   "traffic_source": NCU_TRAFFIC["k_trace"][1],
-                  "kernel": "k_trace + k_retest64 (one rt_trace_closest)",
+                  "kernel": "k_trace (one rt_trace_closest)",
                   "ms": mean_trace_ms, "bytes_per_ray": bytes_per_ray, "algorithmic_bytes": bytes_per_ray * R,
                   "hbm_peak": hbm, "hbm_peak_source": peak_src, "frac_of_hbm": trace_gbs / hbm,
                   "note": "algorithmic bytes = 32 ray + 16 hit + node bytes (32 B per child slot) x nodes + "

@@ -265,8 +265,7 @@ int rt_bvh_export(rt_scene scene, void* stream, int32_t* child, int64_t* leaf_fi
  * tmax); those are traced again in float64 with the same hit rule as the
  * reference definition (Moller-Trumbore, inclusive edges).
  * rays_dev: n rt_ray (16-byte aligned); hits_dev: n rt_hit.  n may be 0.
- * Errors: RT_EINVAL, RT_ENOTBUILT, RT_ENOMEM (first use of a larger n
- * grows the scene's re-test queue), RT_ECUDA. */
+ * Errors: RT_EINVAL, RT_ENOTBUILT, RT_ECUDA. */
 int rt_trace_closest(rt_scene scene, const rt_ray* rays_dev, int64_t n, rt_hit* hits_dev,
                      const rt_trace_params* params, void* stream);
 
@@ -525,8 +524,8 @@ typedef struct {
  * and max_slots concurrent requests (1..64), each on its own stream.  A
  * worker thread admits queued requests in arrival order whenever a slot is
  * free and the pool holds all of the request's buffers (rays, hits, skip and
- * parent arrays per order, re-test scratch: about n * (56 (max_order + 1) + 44)
- * bytes for n rays), so requests of uneven sizes run side by side on the
+ * parent arrays per order, and 44 bytes a ray that are not used any more:
+ * about n * (56 (max_order + 1) + 44) bytes for n rays), so requests of uneven sizes run side by side on the
  * device.  The calling thread's current device is used.
  * Errors: RT_EINVAL, RT_ENOMEM, RT_ECUDA. */
 int rt_session_create(size_t pool_bytes, int max_slots, rt_session* out);
@@ -570,23 +569,11 @@ int rt_session_destroy(rt_session session);
  * rt_trace_closest, for callers that must not let the library allocate
  * device memory: a runtime that manages all device memory through its own
  * pool, or a latency-critical stream where a cudaMalloc (which can
- * synchronise the device) would stall other work.  The scratch for the
- * float64 re-test comes from one fixed array compiled into the library
- * (10 MiB on every GPU that loads it, held until the process exits), not
- * from the scene.
+ * synchronise the device) would stall other work.
  *  - n must not exceed RT_NOALLOC_MAX_RAYS; larger batches return
  *    RT_EINVAL ("split the batch").
- *  - The first call on each device looks up the array's device address
- *    (cudaGetSymbolAddress) with that device current; make that first call
- *    before any stream capture.
- *  - Every call shares the one array: calls whose work overlaps on the GPU
- *    (other streams, other host threads) race with each other.  Issue them
- *    on one stream or order them with events.
  *  - The scene's BVH must already be built (building allocates), and the
  *    device the scene was uploaded on must be current (RT_EINVAL otherwise).
- *  - The array's address is looked up once per device and kept: after a
- *    device reset (cudaDeviceReset), which invalidates every scene, this
- *    call must not be used again in the same process.
  * Errors: RT_EINVAL, RT_ENOTBUILT, RT_ECUDA. */
 int rt_trace_closest_noalloc(rt_scene scene, const rt_ray* rays_dev, int64_t n, rt_hit* hits_dev,
                              const rt_trace_params* params, void* stream);

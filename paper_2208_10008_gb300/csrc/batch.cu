@@ -42,7 +42,7 @@ struct rt_batch_s {
   int* blocks = nullptr;  // reflect block counts
   rt_ray* seg = nullptr;  // visibility segments, transmitter-major
   uint8_t* occl = nullptr;
-  rt::TraceScratch scr;
+  int* flagged = nullptr;  // device: flagged rays of the last walk
   cudaStream_t st = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   cudaGraph_t graph = nullptr;
@@ -131,7 +131,7 @@ void free_batch(rt_batch_s* b) {
     if (b->skip[k]) cudaFree(b->skip[k]);
     if (b->src[k]) cudaFree(b->src[k]);
   }
-  void* p[] = {b->counts, b->blocks, b->seg, b->occl, b->scr.counter, b->scr.queue, b->scr.cand};
+  void* p[] = {b->counts, b->blocks, b->seg, b->occl, b->flagged};
   for (void* q : p)
     if (q) cudaFree(q);
   drop_graph(b);
@@ -168,7 +168,7 @@ cudaError_t enqueue(rt_batch_s* b) {
   L.status = reinterpret_cast<int*>(b->bar + 2);
   L.take = b->take;
   L.timeout_ns = kBarrierTimeoutNs;
-  L.scr = &b->scr;
+  L.flagged = b->flagged;
   L.receive = b->receive ? 1 : 0;
   for (int k = 0; k <= RT_BATCH_MAX_ORDER; ++k) L.delta[k] = b->delta[k];
   if ((e = rt::launch_batch_persistent(b->scene, L, st))) return e;
@@ -283,11 +283,7 @@ static int rt_batch_create_body(rt_scene scene, const rt_batch_desc* d, rt_batch
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);  // off and gp are host temporaries
   }
   if (e == cudaSuccess) e = alloc(&b->blocks, total / 256 + 2);
-  const long long qcap = total > b->n_seg ? total : b->n_seg;
-  if (e == cudaSuccess) e = alloc(&b->scr.counter, 4);
-  if (e == cudaSuccess) e = alloc(&b->scr.queue, qcap);
-  if (e == cudaSuccess) e = alloc(&b->scr.cand, qcap * (rt::kTraceCand + 1));
-  b->scr.cap = qcap;
+  if (e == cudaSuccess) e = alloc(&b->flagged, 1);
   if (e == cudaSuccess && b->n_seg > 0) {
     e = alloc(&b->seg, b->n_seg);
     if (e == cudaSuccess) e = alloc(&b->occl, b->n_seg);
@@ -432,7 +428,7 @@ static int rt_batch_stats_get_body(rt_batch b, void* stream, rt_batch_stats* s) 
     for (int k = 0; k <= b->max_order; ++k) s->received[k] = rc[k];
   }
   int fl = 0;
-  cudaMemcpy(&fl, b->scr.counter, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaMemcpy(&fl, b->flagged, sizeof(int), cudaMemcpyDeviceToHost);
   s->flagged = fl;
   s->segments = b->n_seg;
   unsigned w[4] = {0, 0, 0, 0};

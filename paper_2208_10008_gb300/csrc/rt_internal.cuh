@@ -196,13 +196,7 @@ struct BuildGeom {
 };
 BuildGeom build_geometry(int64_t n_tri, int nsm);
 
-// Per-call trace scratch: counter + queue of flagged ray indices.
-struct TraceScratch {
-  int* counter = nullptr;   // [0] flagged count, [1] status
-  int* queue = nullptr;     // flagged ray indices
-  int* cand = nullptr;      // per queue slot: 1 + kTraceCand ints
-  int64_t cap = 0;
-};
+// Float64 candidates that a walk remembers per ray.
 constexpr int kTraceCand = 8;
 
 // Order-preserving float <-> int map for atomicMin/atomicMax on floats.
@@ -243,12 +237,10 @@ struct SceneDev;  // forward
 
 cudaError_t launch_build(struct ::rt_scene_s* s, const rt_build_params& p, cudaStream_t st);
 cudaError_t launch_trace(struct ::rt_scene_s* s, const rt_ray* rays, int64_t n, rt_hit* hits,
-                         uint8_t* occl, const rt_trace_params* tp, TraceScratch& scr,
-                         cudaStream_t st);
+                         uint8_t* occl, const rt_trace_params* tp, cudaStream_t st);
 // As launch_trace, with the ray count read on the device from n_dev (<= n, the capacity).
 cudaError_t launch_trace_dev(struct ::rt_scene_s* s, const rt_ray* rays, int64_t n, const int* n_dev,
-                             rt_hit* hits, uint8_t* occl, const rt_trace_params* tp, TraceScratch& scr,
-                             cudaStream_t st);
+                             rt_hit* hits, uint8_t* occl, const rt_trace_params* tp, cudaStream_t st);
 cudaError_t launch_gen_rays(int kind, const float* origin, long long param, float tmin, float tmax,
                             rt_ray* rays, long long count, cudaStream_t st);
 // Band width w and in-band step c of the launch order of an n-ray Fibonacci
@@ -371,7 +363,7 @@ struct BatchLaunch {
   int* status;
   int* take;        // [RT_BATCH_MAX_ORDER + 2]
   long long timeout_ns;
-  TraceScratch* scr;
+  int* flagged;     // rays that went through the float64 pass in the last walk
   // reception (Eq. 4) afterwards: every bounced ray takes its parent's delta
   int receive;
   float* delta[RT_BATCH_MAX_ORDER + 1];         // per ray: its transmitter's delta (order 0 given)
@@ -424,8 +416,6 @@ struct rt_scene_s {
   int* top_ready = nullptr;         // [cap_c] epoch stamp of each published item
   rt::BuildGeom geom{};             // geometry the buffers were sized for
   rt::BuildCtl* ctl = nullptr;
-  rt::TraceScratch scratch;     // default trace scratch
-  rt::TraceScratch host_scr[2]; // scratch of the host-buffer pipeline
   int* reflect_blocks = nullptr; // per-block counts of rt_reflect
   int64_t reflect_blocks_cap = 0;
   rt_ray* stage_rays[2] = {nullptr, nullptr};

@@ -95,9 +95,7 @@ __global__ void k_child_refs(const rt::WNode* __restrict__ w4, const rt::WNode8*
 void free_scene_buffers(rt_scene_s* s) {
   void* ptrs[] = {s->tri_in, s->idx[0], s->idx[1], s->rec[0], s->rec[1], s->node2, s->wide, s->link2, s->epoch,
                   s->tri_leaf, s->qa, s->qa_ready, s->top_task, s->top_done, s->top_bins, s->top_ccnt,
-                  s->top_scnt, s->top_item, s->top_plan, s->top_ready, s->ctl, s->scratch.counter, s->scratch.queue, s->scratch.cand,
-                  s->host_scr[0].counter, s->host_scr[0].queue, s->host_scr[0].cand,
-                  s->host_scr[1].counter, s->host_scr[1].queue, s->host_scr[1].cand, s->reflect_blocks,
+                  s->top_scnt, s->top_item, s->top_plan, s->top_ready, s->ctl, s->reflect_blocks,
                   s->stage_rays[0], s->stage_rays[1], s->stage_hits[0], s->stage_hits[1], s->sel, s->sel_cnt,
                   s->qwide, s->wide8};
   for (void* p : ptrs)
@@ -183,20 +181,6 @@ int alloc_capacity(rt_scene_s* s, int64_t m) {
   if (!s->ctl) RT_CUDA(cudaMalloc((void**)&s->ctl, sizeof(rt::BuildCtl)), "alloc control block");
   s->geom = g;
   s->cap_tri = m;
-  return RT_OK;
-}
-
-int ensure_scratch(rt::TraceScratch& scr, int64_t n) {
-  if (scr.counter && scr.cap >= n) return RT_OK;
-  if (!scr.counter) RT_CUDA(cudaMalloc((void**)&scr.counter, 4 * sizeof(int)), "alloc trace counter");
-  if (scr.queue) cudaFree(scr.queue);
-  if (scr.cand) cudaFree(scr.cand);
-  scr.queue = nullptr;
-  scr.cand = nullptr;
-  int64_t cap = n < 1024 ? 1024 : n;
-  RT_CUDA(cudaMalloc((void**)&scr.queue, cap * sizeof(int)), "alloc re-test queue");
-  RT_CUDA(cudaMalloc((void**)&scr.cand, cap * (rt::kTraceCand + 1) * sizeof(int)), "alloc re-test candidates");
-  scr.cap = cap;
   return RT_OK;
 }
 
@@ -518,9 +502,7 @@ static int trace_common(rt_scene s, const rt_ray* rays, int64_t n, rt_hit* hits,
   if (params && (params->flags & RT_QUANTIZED_NODES) && !s->q_built)
     return fail(RT_EINVAL, "RT_QUANTIZED_NODES needs a build with quantize = 1");
   if (!s->built) return fail(RT_ENOTBUILT, "BVH not built");
-  int r = ensure_scratch(s->scratch, n);
-  if (r) return r;
-  RT_CUDA(rt::launch_trace(s, rays, n, hits, occl, params, s->scratch, (cudaStream_t)stream), "launch trace");
+  RT_CUDA(rt::launch_trace(s, rays, n, hits, occl, params, (cudaStream_t)stream), "launch trace");
   return RT_OK;
 }
 
@@ -624,8 +606,6 @@ int rt_trace_closest_host(rt_scene s, const rt_ray* rays_host, int64_t n, rt_hit
   }
   for (int k = 0; k < 2; ++k) {
     if (!s->host_streams[k]) RT_CUDA(cudaStreamCreateWithFlags(&s->host_streams[k], cudaStreamNonBlocking), "create stream");
-    int r = ensure_scratch(s->host_scr[k], chunk);
-    if (r) return r;
   }
   // the ray copies start at once (they read only the caller's host buffer);
   // the traces wait for everything already queued on the caller's stream
@@ -660,7 +640,7 @@ int rt_trace_closest_host(rt_scene s, const rt_ray* rays_host, int64_t n, rt_hit
                                     cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && c < 2) e = cudaStreamWaitEvent(st, ev, 0);
     rt_hit* out = hits_mapped ? hits_mapped + off : s->stage_hits[k];
-    if (e == cudaSuccess) e = rt::launch_trace(s, s->stage_rays[k], cnt, out, nullptr, &tp, s->host_scr[k], st);
+    if (e == cudaSuccess) e = rt::launch_trace(s, s->stage_rays[k], cnt, out, nullptr, &tp, st);
     if (e == cudaSuccess && !hits_mapped)
       e = cudaMemcpyAsync(hits_host + off, s->stage_hits[k], cnt * sizeof(rt_hit), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) {

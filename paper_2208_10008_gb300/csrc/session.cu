@@ -176,7 +176,6 @@ struct Req {
   int* src[RT_BATCH_MAX_ORDER + 1] = {};
   int* counts = nullptr;
   int* blocks = nullptr;
-  rt::TraceScratch scr;
 };
 
 struct Slot {
@@ -193,7 +192,7 @@ size_t request_bytes(long long n, int orders) {
   size_t b = per_order * (size_t)(orders + 1);
   b += 64 + (size_t)(RT_BATCH_MAX_ORDER + 1) * sizeof(int);      // counts
   b += ((size_t)n / 256 + 2) * sizeof(int);                       // reflect blocks
-  b += 64 + (size_t)n * sizeof(int) * (1 + rt::kTraceCand + 1);    // trace counter, queue, candidates
+  b += 64 + (size_t)n * sizeof(int) * 10;                         // not used: a request's size decides which are refused
   return b + 64 * 256;                                            // alignment slack (<= 48 arrays)
 }
 
@@ -249,17 +248,13 @@ cudaError_t start(rt_session_s* S, Req* q, Slot& sl) {
   }
   q->counts = carve<int>(base, &at, RT_BATCH_MAX_ORDER + 1);
   q->blocks = carve<int>(base, &at, q->n / 256 + 2);
-  q->scr.counter = carve<int>(base, &at, 16);
-  q->scr.queue = carve<int>(base, &at, q->n);
-  q->scr.cand = carve<int>(base, &at, (size_t)q->n * (rt::kTraceCand + 1));
-  q->scr.cap = q->n;
   cudaError_t e;
   cudaStream_t st = sl.st;
   if ((e = cudaMemsetAsync(q->counts, 0, (RT_BATCH_MAX_ORDER + 1) * sizeof(int), st))) return e;
   if ((e = rt::launch_gen_rays(q->r.dir_kind, q->r.tx, q->r.param, 0.f, q->r.tmax, q->rays[0], q->n, st)))
     return e;
   rt_trace_params tp{};
-  if ((e = rt::launch_trace_dev(scene, q->rays[0], q->n, nullptr, q->hits[0], nullptr, &tp, q->scr, st))) return e;
+  if ((e = rt::launch_trace_dev(scene, q->rays[0], q->n, nullptr, q->hits[0], nullptr, &tp, st))) return e;
   for (int k = 1; k <= orders; ++k) {
     const int* prev = k == 1 ? nullptr : q->counts + (k - 1);
     if ((e = rt::launch_reflect(scene, q->rays[k - 1], q->hits[k - 1], q->n, prev, q->rays[k], q->skip[k], q->src[k],
@@ -267,7 +262,7 @@ cudaError_t start(rt_session_s* S, Req* q, Slot& sl) {
       return e;
     rt_trace_params tk{};
     tk.skip_tri_dev = q->skip[k];
-    if ((e = rt::launch_trace_dev(scene, q->rays[k], q->n, q->counts + k, q->hits[k], nullptr, &tk, q->scr, st)))
+    if ((e = rt::launch_trace_dev(scene, q->rays[k], q->n, q->counts + k, q->hits[k], nullptr, &tk, st)))
       return e;
   }
   if (q->r.hits_host) {

@@ -22,12 +22,10 @@
 //     2013), two-sided, plus a forward error bound E on its three edge
 //     functions.  Signs settled beyond E give a certain hit or miss; anything
 //     else, a second hit within the error window of the best one, a hit near
-//     tmin / tmax, or a stack overflow marks the ray for k_retest64.
-// k_retest64 (float64, flagged rays only)
-//   * rays with a candidate list: a group of lanes per ray (a warp when few
-//     rays are flagged, one lane when many are) applies the float64 rule to
-//     the candidates and a group reduction keeps the nearest; when the
-//     list overflowed, one thread per ray does a stackless walk of the
+//     tmin / tmax, or a stack overflow marks the ray for the float64 pass.
+// retest_ray (float64, flagged rays only, at the end of their walk)
+//   * applies the float64 rule to the candidates the walk remembered and keeps
+//     the nearest; when the list overflowed, a stackless walk of the
 //     binary tree (parent links) with the same conservative float32 box test
 //     culled at the float64 best distance, and for every triangle the
 //     float32 bound does not prove missed, the reference hit rule:
@@ -48,7 +46,6 @@ namespace {
 
 constexpr int kTraceBlock = 128;
 constexpr int kStack = 64;  // default depth of the walk's stack
-constexpr int kRetestBlock = 128;
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr float kU = 5.9604645e-08f;   // unit roundoff of float32, 2^-24
 constexpr float kWiden = 1e-6f;        // relative widening of box intervals
@@ -361,21 +358,6 @@ __device__ __forceinline__ void cswap(float& ta, int& ra, float& tb, int& rb) {
   }
 }
 
-__device__ __forceinline__ int enqueue_flag(int* counter, int* queue, int qcap, int i) {
-  unsigned m = __activemask();
-  int lane = threadIdx.x & 31;
-  int leader = __ffs(m) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(counter, __popc(m));
-  base = __shfl_sync(m, base, leader);
-  int s = base + __popc(m & ((1u << lane) - 1u));
-  if (s < qcap) {
-    queue[s] = i;
-    return s;
-  }
-  return -1;
-}
-
 struct TraceArgs {
   const WNode* wide;
   const WNode8* wide8;   // 8-wide nodes (walk with kW = 8)
@@ -393,12 +375,169 @@ struct TraceArgs {
   uint8_t* occl;
   const int32_t* skip;
   uint32_t* stats;
-  int* counter;
-  int* queue;
-  int* cand;  // per queue slot: count (-1 = walk the whole tree) + kCand leaf positions
-  int qcap;
+  int* counter;  // nullable: flagged rays are counted here
+  int retest;    // 1: flagged rays get the float64 pass
 };
 
+// ---------------------------------------------------------------- float64
+struct D3 {
+  double x, y, z;
+};
+__device__ __forceinline__ D3 dsub3(D3 a, D3 b) {
+  return {__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y), __dsub_rn(a.z, b.z)};
+}
+// (a.x*b.x + a.y*b.y) + a.z*b.z, rounded at every step
+__device__ __forceinline__ double ddot(D3 a, D3 b) {
+  double s = __dmul_rn(a.x, b.x);
+  s = __dadd_rn(s, __dmul_rn(a.y, b.y));
+  s = __dadd_rn(s, __dmul_rn(a.z, b.z));
+  return s;
+}
+__device__ __forceinline__ D3 dcross(D3 a, D3 b) {
+  return {__dsub_rn(__dmul_rn(a.y, b.z), __dmul_rn(a.z, b.y)),
+          __dsub_rn(__dmul_rn(a.z, b.x), __dmul_rn(a.x, b.z)),
+          __dsub_rn(__dmul_rn(a.x, b.y), __dmul_rn(a.y, b.x))};
+}
+
+// Moller-Trumbore, the reference hit rule (see file header).
+__device__ bool mt64(D3 o, D3 d, D3 v0, D3 v1, D3 v2, double* t, double* u, double* v) {
+  D3 e1 = dsub3(v1, v0), e2 = dsub3(v2, v0);
+  D3 p = dcross(d, e2);
+  double det = ddot(e1, p);
+  // the squares tell a determinant well above the limit (their rounding is
+  // below 1e-14 of the product); only near it are the three roots taken
+  const double q1 = ddot(e1, e1), q2 = ddot(e2, e2), qd = ddot(d, d);
+  if (!(__dmul_rn(det, det) > __dmul_rn(1.0001e-28, __dmul_rn(__dmul_rn(q1, q2), qd)))) {
+    double n1 = __dsqrt_rn(q1), n2 = __dsqrt_rn(q2), nd = __dsqrt_rn(qd);
+    double lim = __dmul_rn(1e-14, __dmul_rn(__dmul_rn(n1, n2), nd));
+    if (fabs(det) <= lim) return false;
+  }
+  double inv = __ddiv_rn(1.0, det);
+  D3 s = dsub3(o, v0);
+  double uu = __dmul_rn(ddot(s, p), inv);
+  if (uu < 0.0 || uu > 1.0) return false;
+  D3 q = dcross(s, e1);
+  double vv = __dmul_rn(ddot(d, q), inv);
+  if (vv < 0.0 || __dadd_rn(uu, vv) > 1.0) return false;
+  *t = __dmul_rn(ddot(e2, q), inv);
+  *u = uu;
+  *v = vv;
+  return true;
+}
+
+// The float64 pass of ray i, which the float32 walk flagged: its candidates
+// (leaf positions cand[0 .. nc)) by the float64 rule, the nearest kept, the
+// lowest id on ties; without a complete list (nc < 0) every triangle that the
+// float32 bound does not prove missed.  Called by the flagged lanes at the
+// end of their walk, a few dozen of 655,362 on the medium city, while other
+// warps walk: as a kernel of its own behind the walk (queue, counter, a group
+// of lanes per ray) it took 12 us of the 110 us of a trace, most of them its
+// launch and its chain of dependent loads and float64 operations.  Not
+// inlined, so that the walk's registers are its own.
+template <bool kAny>
+__device__ __noinline__ void retest_ray(const TraceArgs& A, const float4* r4, const int skip, const int* cand,
+                                        const int nc, float4* hit, uint8_t* occl) {
+  const float4 ra = r4[0], rb = r4[1];
+  const RayPre r = setup_ray(ra, rb);
+  const D3 o{ra.x, ra.y, ra.z}, d{rb.x, rb.y, rb.z};
+  const double tmin = ra.w, tmax = rb.w;
+  double bt = INFINITY, bu = 0.0, bv = 0.0;
+  int bid = -1, bpos = -1;
+  bool any = false;
+  auto test = [&](int pos, float4 va, float4 vb, float4 vc) {
+    double t, u, v;
+    if (mt64(o, d, D3{va.x, va.y, va.z}, D3{vb.x, vb.y, vb.z}, D3{vc.x, vc.y, vc.z}, &t, &u, &v) && t > tmin &&
+        t < tmax) {
+      any = true;
+      const int id = __float_as_int(va.w);
+      if (t < bt || (t == bt && (bid < 0 || id < bid))) {
+        bt = t;
+        bid = id;
+        bpos = pos;
+        bu = u;
+        bv = v;
+      }
+    }
+  };
+#pragma unroll 1
+  for (int q = 0; q < nc; ++q) {
+    const float4* tp = A.tris + 3 * (size_t)cand[q];
+    const float4 va = tp[0];
+    if (__float_as_int(va.w) != skip) test(cand[q], va, tp[1], tp[2]);
+  }
+  if (nc < 0 && r.valid) {
+    // A stackless walk of the binary tree (parent links), so that any depth
+    // works.  Boxes use the same widened float32 slab test as the walk, culled
+    // at the float64 best distance rounded up.
+    auto test_leaf = [&](int ref) {
+      const int first = leaf_first(ref), count = leaf_count(ref);
+      for (int k = 0; k < count && !(kAny && any); ++k) {
+        const float4* tp = A.tris + 3 * (size_t)(first + k);
+        const float4 va = tp[0], vb = tp[1], vc = tp[2];
+        if (__float_as_int(va.w) == skip) continue;
+        if (tri_test(r, va, vb, vc).cls == 0) continue;  // certain miss
+        test(first + k, va, vb, vc);
+      }
+    };
+    const int root = *A.root_ref;
+    if (root >= A.n_tri - 1) {
+      // no usable tree: nothing to walk
+    } else if (root < 0) {
+      if (root != INT_MIN) test_leaf(root);
+    } else {
+      int node = root, s = 0;  // s: next child of `node` to try (2: done)
+      for (long long guard = 0; guard < (1ll << 32); ++guard) {
+        if (s < 2) {
+          const Node2* nd = A.node2 + node;
+          const float4 lo = s == 0 ? nd->a_lo : nd->b_lo, hi = s == 0 ? nd->a_hi : nd->b_hi;
+          float bf = (float)fmin(bt, tmax);
+          bf = bf + fabsf(bf) * 2e-6f;
+          ++s;
+          if (!slab1(lo, hi, r, bf)) continue;
+          const int ref = __float_as_int(lo.w);
+          if (ref >= 0) {
+            if (ref < A.n_tri - 1) {  // a link the build never wrote is skipped
+              node = ref;
+              s = 0;
+            }
+            continue;
+          }
+          test_leaf(ref);
+          if (kAny && any) break;
+          continue;
+        }
+        if (node == root) break;
+        const int p = A.link2[node].x;
+        if (p < 0 || p >= A.n_tri - 1) break;
+        s = __float_as_int(A.node2[p].a_lo.w) == node ? 1 : 2;
+        node = p;
+      }
+    }
+  }
+  if (kAny) {
+    *occl = any ? 1 : 0;
+    return;
+  }
+  float4 out = make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
+  if (bid >= 0) {
+    out = make_float4((float)bt, __int_as_float(bid), (float)bu, (float)bv);
+    // The record is a function of the ray and the winning triangle only:
+    // where the float32 test certifies the winner, report exactly what
+    // the float32 walk reports for it (so the result never depends on
+    // whether this tree's walk flagged the ray).
+    const float4* tp = A.tris + 3 * (size_t)bpos;
+    const float4 va = tp[0], vb = tp[1], vc = tp[2];
+    const TriRes h = tri_test(r, va, vb, vc);
+    if (h.cls == 1 && h.t > r.tmin && h.t < r.tmax) {
+      float t = h.t;
+      if (h.err > 0.25f * (kTieRel * h.t + 1e-6f)) t = refine_t(r, rb.x, rb.y, rb.z, va, vb, vc);
+      out = make_float4(t, __int_as_float(bid), h.u, h.v);
+    }
+  }
+  *hit = out;
+}
+
+// ---------------------------------------------------------------- the walk
 // The float32 walk of ray i (the whole of Fig. 4 for one ray): results,
 // statistics and the flag for the float64 pass.  Called by whole warps;
 // lanes without a ray pass live = false.  A lane visits the same boxes and
@@ -585,12 +724,30 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       bound = fminf(r.tmax, t1 + kTieRel * t1 + e1);
     }
   }
+  if (kAny) {
+    if (done) flag = false;
+  } else if (t2 < INFINITY && t2 <= t1 + kTieRel * t1 + e1 + e2) {
+    flag = true;
+  }
+  if (A.counter) {
+    const unsigned m = __ballot_sync(kFullMask, flag);
+    if ((threadIdx.x & 31) == 0 && m) atomicAdd(A.counter, __popc(m));
+  }
   if (!live) return;
+  if (kStats && A.stats) {
+    A.stats[2 * (size_t)i] = n_nodes;
+    A.stats[2 * (size_t)i + 1] = n_tris;
+  }
+  if (flag && A.retest) {
+    int w = 0;
+    for (int q = 0; q < nc; ++q)
+      if (clo[q] <= bound) cpos[w++] = cpos[q];
+    retest_ray<kAny>(A, r4, skip, cpos, walk_all ? -1 : w, reinterpret_cast<float4*>(hits) + i, occl + i);
+    return;
+  }
   if (kAny) {
     occl[i] = done ? 1 : 0;
-    if (done) flag = false;
   } else {
-    if (t2 < INFINITY && t2 <= t1 + kTieRel * t1 + e1 + e2) flag = true;
     if (id1 >= 0 && e1 > 0.25f * (kTieRel * t1 + 1e-6f)) {
       // the float32 distance is not certified inside the tolerance: recompute it
       const float4* tp = A.tris + 3 * (size_t)pos1;
@@ -600,21 +757,6 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
     float4 out = id1 >= 0 ? make_float4(t1, __int_as_float(id1), bu, bv)
                           : make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
     reinterpret_cast<float4*>(hits)[i] = out;
-  }
-  if (kStats && A.stats) {
-    A.stats[2 * (size_t)i] = n_nodes;
-    A.stats[2 * (size_t)i + 1] = n_tris;
-  }
-  if (flag) {
-    const int slot = enqueue_flag(A.counter, A.queue, A.qcap, i);
-    if (slot >= 0) {
-      int* c = A.cand + (size_t)slot * (kCand + 1);
-      int w = 0;
-      if (!walk_all)
-        for (int q = 0; q < nc; ++q)
-          if (clo[q] <= bound) c[1 + w++] = cpos[q];
-      c[0] = walk_all ? -1 : w;
-    }
   }
 }
 
@@ -635,268 +777,22 @@ __global__ void __launch_bounds__(kTile, walk_ctas<kAny, kStats, kTile, kSD, kQu
   walk_one<kAny, kStats, kSD, kQuant, kW>(A, i, live, A.rays, A.hits, A.occl, A.skip);
 }
 
-// ---------------------------------------------------------------- float64
-struct D3 {
-  double x, y, z;
-};
-__device__ __forceinline__ D3 dsub3(D3 a, D3 b) {
-  return {__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y), __dsub_rn(a.z, b.z)};
-}
-// (a.x*b.x + a.y*b.y) + a.z*b.z, rounded at every step
-__device__ __forceinline__ double ddot(D3 a, D3 b) {
-  double s = __dmul_rn(a.x, b.x);
-  s = __dadd_rn(s, __dmul_rn(a.y, b.y));
-  s = __dadd_rn(s, __dmul_rn(a.z, b.z));
-  return s;
-}
-__device__ __forceinline__ D3 dcross(D3 a, D3 b) {
-  return {__dsub_rn(__dmul_rn(a.y, b.z), __dmul_rn(a.z, b.y)),
-          __dsub_rn(__dmul_rn(a.z, b.x), __dmul_rn(a.x, b.z)),
-          __dsub_rn(__dmul_rn(a.x, b.y), __dmul_rn(a.y, b.x))};
-}
-
-// Moller-Trumbore, the reference hit rule (see file header).
-__device__ bool mt64(D3 o, D3 d, D3 v0, D3 v1, D3 v2, double* t, double* u, double* v) {
-  D3 e1 = dsub3(v1, v0), e2 = dsub3(v2, v0);
-  D3 p = dcross(d, e2);
-  double det = ddot(e1, p);
-  double n1 = __dsqrt_rn(ddot(e1, e1)), n2 = __dsqrt_rn(ddot(e2, e2)), nd = __dsqrt_rn(ddot(d, d));
-  double lim = __dmul_rn(1e-14, __dmul_rn(__dmul_rn(n1, n2), nd));
-  if (fabs(det) <= lim) return false;
-  double inv = __ddiv_rn(1.0, det);
-  D3 s = dsub3(o, v0);
-  double uu = __dmul_rn(ddot(s, p), inv);
-  if (uu < 0.0 || uu > 1.0) return false;
-  D3 q = dcross(s, e1);
-  double vv = __dmul_rn(ddot(d, q), inv);
-  if (vv < 0.0 || __dadd_rn(uu, vv) > 1.0) return false;
-  *t = __dmul_rn(ddot(e2, q), inv);
-  *u = uu;
-  *v = vv;
-  return true;
-}
-
-// Flagged rays with a candidate list: a group of G lanes each (G a power of
-// two, the widest up to 32 that still gives every flagged ray its own group
-// in this grid, so a handful of rays gets a warp each and a flood gets a
-// thread each); lane q of a group tests candidates q, q + G, ... with the
-// float64 rule and a reduction over the group keeps the nearest (lowest id on
-// ties, the same minimum whatever G is).  Rays without a complete list: one
-// thread each walks the tree.
-// The float64 pass over every flagged ray, by threads tid of nthreads
-// (nthreads a multiple of 32, whole warps).
-template <bool kAny>
-__device__ void retest_all(const TraceArgs& A, const int tid, const int nthreads, const rt_ray* __restrict__ rays,
-                           rt_hit* __restrict__ hits, uint8_t* __restrict__ occl,
-                           const int32_t* __restrict__ skip_ids) {
-  const int nflag = min(*(volatile int*)A.counter, A.qcap);
-  if (nflag <= 0) return;
-  int lg = 5;
-  while (lg > 0 && ((long long)nflag << lg) > nthreads) --lg;
-  const int lane = threadIdx.x & 31, sub = lane & ((1 << lg) - 1);
-  const int ngroups = nthreads >> lg;
-  // jw: the first ray of this warp's groups; the loop is uniform over the warp
-  for (int jw = (tid & ~31) >> lg; jw < nflag; jw += ngroups) {
-    const int j = jw + (lane >> lg);
-    const bool live = j < nflag;
-    const int* cl = A.cand + (size_t)(live ? j : 0) * (kCand + 1);
-    const int ncand = live ? cl[0] : -1;
-    const int i = live ? A.queue[j] : 0;
-    const float4* r4 = reinterpret_cast<const float4*>(rays) + 2 * (size_t)i;
-    float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
-    if (ncand > 0) {
-      ra = r4[0];
-      rb = r4[1];
-    }
-    const D3 o{ra.x, ra.y, ra.z}, d{rb.x, rb.y, rb.z};
-    const double tmin = ra.w, tmax = rb.w;
-    const int skip = (ncand > 0 && skip_ids) ? skip_ids[i] : -1;
-    double bt = INFINITY, bu = 0.0, bv = 0.0;
-    int bid = INT_MAX, bpos = -1;
-    for (int q = sub; q < ncand; q += 1 << lg) {
-      const int pos = cl[1 + q];
-      const float4* tp = A.tris + 3 * (size_t)pos;
-      const float4 va = tp[0], vb = tp[1], vc = tp[2];
-      const int id = __float_as_int(va.w);
-      double t, u, v;
-      if (id != skip && mt64(o, d, D3{va.x, va.y, va.z}, D3{vb.x, vb.y, vb.z}, D3{vc.x, vc.y, vc.z}, &t, &u, &v) &&
-          t > tmin && t < tmax && (t < bt || (t == bt && id < bid))) {
-        bt = t;
-        bid = id;
-        bpos = pos;
-        bu = u;
-        bv = v;
-      }
-    }
-    for (int off = (1 << lg) >> 1; off > 0; off >>= 1) {
-      const double ot = __shfl_xor_sync(kFullMask, bt, off);
-      const int oid = __shfl_xor_sync(kFullMask, bid, off);
-      const int opos = __shfl_xor_sync(kFullMask, bpos, off);
-      const double ou = __shfl_xor_sync(kFullMask, bu, off), ov = __shfl_xor_sync(kFullMask, bv, off);
-      if (ot < bt || (ot == bt && oid < bid)) {
-        bt = ot;
-        bid = oid;
-        bpos = opos;
-        bu = ou;
-        bv = ov;
-      }
-    }
-    if (ncand < 0 || sub != 0) continue;  // a whole-tree walk is done below
-    if (ncand == 0) {
-      ra = r4[0];
-      rb = r4[1];
-    }
-    const RayPre r = setup_ray(ra, rb);
-    if (kAny) {
-      occl[i] = bid != INT_MAX ? 1 : 0;
-    } else {
-      float4 out = make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
-      if (bid != INT_MAX) {
-        out = make_float4((float)bt, __int_as_float(bid), (float)bu, (float)bv);
-        // The record is a function of the ray and the winning triangle only:
-        // where the float32 test certifies the winner, report exactly what
-        // the float32 walk reports for it (so the result never depends on
-        // whether this tree's walk flagged the ray).
-        const float4* tp = A.tris + 3 * (size_t)bpos;
-        const float4 va = tp[0], vb = tp[1], vc = tp[2];
-        const TriRes h = tri_test(r, va, vb, vc);
-        if (h.cls == 1 && h.t > r.tmin && h.t < r.tmax) {
-          float t = h.t;
-          if (h.err > 0.25f * (kTieRel * h.t + 1e-6f)) t = refine_t(r, rb.x, rb.y, rb.z, va, vb, vc);
-          out = make_float4(t, __int_as_float(bid), h.u, h.v);
-        }
-      }
-      reinterpret_cast<float4*>(hits)[i] = out;
-    }
-  }
-  // rays without a complete candidate list: one thread each walks the tree
-  for (int j = tid; j < nflag; j += nthreads) {
-    const int i = A.queue[j];
-    const float4* r4 = reinterpret_cast<const float4*>(rays) + 2 * (size_t)i;
-    const float4 ra = r4[0], rb = r4[1];
-    const RayPre r = setup_ray(ra, rb);
-    const D3 o{ra.x, ra.y, ra.z}, d{rb.x, rb.y, rb.z};
-    const double tmin = ra.w, tmax = rb.w;
-    const int skip = skip_ids ? skip_ids[i] : -1;
-    double bt = INFINITY, bu = 0.0, bv = 0.0;
-    int bid = -1, bpos = -1;
-    bool any = false;
-    const int* cl = A.cand + (size_t)j * (kCand + 1);
-    const int ncand = cl[0];
-    if (ncand >= 0) continue;  // done by a warp above
-    // Without a complete candidate list: a stackless walk of the binary tree
-    // (parent links), so that any depth works.  Boxes use the same widened
-    // float32 slab test as k_trace, culled at the float64 best distance
-    // rounded up; triangles the float32 bound proves missed are skipped,
-    // every other one goes through the float64 rule.
-    auto test_leaf = [&](int ref) {
-      const int first = leaf_first(ref), count = leaf_count(ref);
-      for (int k = 0; k < count && !(kAny && any); ++k) {
-        const float4* tp = A.tris + 3 * (size_t)(first + k);
-        const float4 va = tp[0], vb = tp[1], vc = tp[2];
-        const int id = __float_as_int(va.w);
-        if (id == skip) continue;
-        if (tri_test(r, va, vb, vc).cls == 0) continue;  // certain miss
-        double t, u, v;
-        if (mt64(o, d, D3{va.x, va.y, va.z}, D3{vb.x, vb.y, vb.z}, D3{vc.x, vc.y, vc.z}, &t, &u, &v) && t > tmin &&
-            t < tmax) {
-          any = true;
-          if (t < bt || (t == bt && (bid < 0 || id < bid))) {
-            bt = t;
-            bid = id;
-            bpos = first + k;
-            bu = u;
-            bv = v;
-          }
-        }
-      }
-    };
-    if (r.valid) {
-      const int root = *A.root_ref;
-      if (root >= A.n_tri - 1) {
-        // no usable tree: nothing to walk
-      } else if (root < 0) {
-        if (root != INT_MIN) test_leaf(root);
-      } else {
-        int node = root, s = 0;  // s: next child of `node` to try (2: done)
-        for (long long guard = 0; guard < (1ll << 32); ++guard) {
-          if (s < 2) {
-            const Node2* nd = A.node2 + node;
-            const float4 lo = s == 0 ? nd->a_lo : nd->b_lo, hi = s == 0 ? nd->a_hi : nd->b_hi;
-            float bf = (float)fmin(bt, tmax);
-            bf = bf + fabsf(bf) * 2e-6f;
-            ++s;
-            if (!slab1(lo, hi, r, bf)) continue;
-            const int ref = __float_as_int(lo.w);
-            if (ref >= 0) {
-              if (ref < A.n_tri - 1) {  // a link the build never wrote is skipped
-                node = ref;
-                s = 0;
-              }
-              continue;
-            }
-            test_leaf(ref);
-            if (kAny && any) break;
-            continue;
-          }
-          if (node == root) break;
-          const int p = A.link2[node].x;
-          if (p < 0 || p >= A.n_tri - 1) break;
-          s = __float_as_int(A.node2[p].a_lo.w) == node ? 1 : 2;
-          node = p;
-        }
-      }
-    }
-    if (kAny) {
-      occl[i] = any ? 1 : 0;
-    } else {
-      float4 out = make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
-      if (bid >= 0) {
-        out = make_float4((float)bt, __int_as_float(bid), (float)bu, (float)bv);
-        // The record is a function of the ray and the winning triangle only:
-        // where the float32 test certifies the winner, report exactly what
-        // the float32 walk reports for it (so the result never depends on
-        // whether this tree's walk flagged the ray).
-        const float4* tp = A.tris + 3 * (size_t)bpos;
-        const float4 va = tp[0], vb = tp[1], vc = tp[2];
-        const TriRes h = tri_test(r, va, vb, vc);
-        if (h.cls == 1 && h.t > r.tmin && h.t < r.tmax) {
-          float t = h.t;
-          if (h.err > 0.25f * (kTieRel * h.t + 1e-6f)) t = refine_t(r, rb.x, rb.y, rb.z, va, vb, vc);
-          out = make_float4(t, __int_as_float(bid), h.u, h.v);
-        }
-      }
-      reinterpret_cast<float4*>(hits)[i] = out;
-    }
-  }
-}
-
-// Launched as a programmatic dependent of the walk: its CTAs are placed as
-// the walk's last CTAs retire and wait here until the walk's results are
-// visible.
-template <bool kAny>
-__global__ void __launch_bounds__(kRetestBlock) k_retest64(TraceArgs A) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  retest_all<kAny>(A, blockIdx.x * kRetestBlock + threadIdx.x, gridDim.x * kRetestBlock, A.rays, A.hits, A.occl,
-                   A.skip);
-}
-
 // ---------------------------------------------------------------- one launch for a whole batch
 // Every reflection order of a batch (Sec. III.B: trace, bounce, trace the
 // bounced rays, until the order limit) and the visibility segments in one
 // cooperative launch: the CTAs stay resident and step through the phases
 // together, separated by grid barriers:
-//   for each order k: walk (float32) -> barrier -> float64 pass of the flagged
-//   rays -> barrier -> survivors per 32-ray chunk -> barrier -> offsets
-//   (stable, in ray order) -> barrier -> bounce into order k + 1 -> barrier;
-//   then the segments: walk (any hit) -> barrier -> float64 pass.
-// The walk, the float64 pass and the bounce are the same device code as the
+//   for each order k: walk (the flagged rays' float64 pass with it) ->
+//   barrier -> survivors per 32-ray chunk -> barrier -> offsets (stable, in
+//   ray order) -> barrier -> bounce into order k + 1 -> barrier;
+//   then the segments: walk (any hit).
+// The walk and the bounce are the same device code as the
 // separate kernels (rt_trace_closest, rt_reflect), so every order's rays,
 // hits and parent indices are the same bits.  A barrier waits at most
 // timeout_ns (global timer); when it runs out the status word is set and
 // every CTA leaves.
 struct PersistArgs {
-  TraceArgs T;           // scene arrays and the float64 pass's scratch
+  TraceArgs T;           // scene arrays and the count of flagged rays
   const float4* tri_in;  // input-order triangles (bounces)
   int max_order;
   int n0;
@@ -993,7 +889,6 @@ template <int kW>
 __global__ void __launch_bounds__(kPersistBlock, kPersistMinBlocks) k_batch(const __grid_constant__ PersistArgs P) {
   __shared__ int red[kPersistBlock / 32];
   __shared__ int carry;
-  const int nth = gridDim.x * kPersistBlock;
   const int tid = blockIdx.x * kPersistBlock + threadIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kWarps = kPersistBlock / 32;
@@ -1005,11 +900,9 @@ __global__ void __launch_bounds__(kPersistBlock, kPersistMinBlocks) k_batch(cons
     const int* skip = k ? P.skip[k] : nullptr;
     walk_phase<false, kW>(A, P.take + k, n, rays, hits, nullptr, skip);
     if (!grid_sync(P)) return;
-    retest_all<false>(A, tid, nth, rays, hits, nullptr, skip);
-    if (!grid_sync(P)) return;
     if (k == P.max_order) break;
     // survivors of the bounce per 32-ray chunk; CTA b owns a contiguous run of chunks
-    if (tid == 0) *A.counter = 0;  // the next order's flags (this order's float64 pass is done)
+    if (tid == 0) *A.counter = 0;  // the next order's flags
     const int nch = (n + 31) / 32, per = (nch + (int)gridDim.x - 1) / (int)gridDim.x;
     const int c0 = min(nch, (int)blockIdx.x * per), c1 = min(nch, c0 + per);
     if (threadIdx.x == 0) carry = 0;
@@ -1090,8 +983,6 @@ __global__ void __launch_bounds__(kPersistBlock, kPersistMinBlocks) k_batch(cons
     if (tid == 0) *A.counter = 0;
     if (!grid_sync(P)) return;
     walk_phase<true, kW>(A, P.take + RT_BATCH_MAX_ORDER + 1, P.n_seg, P.seg, nullptr, P.occl, nullptr);
-    if (!grid_sync(P)) return;
-    retest_all<true>(A, tid, nth, P.seg, nullptr, P.occl, nullptr);
   }
 }
 
@@ -1109,8 +1000,8 @@ int sm_count_t() {
 }  // namespace
 
 cudaError_t launch_trace(rt_scene_s* s, const rt_ray* rays, int64_t n, rt_hit* hits, uint8_t* occl,
-                         const rt_trace_params* tp, TraceScratch& scr, cudaStream_t st) {
-  return launch_trace_dev(s, rays, n, nullptr, hits, occl, tp, scr, st);
+                         const rt_trace_params* tp, cudaStream_t st) {
+  return launch_trace_dev(s, rays, n, nullptr, hits, occl, tp, st);
 }
 
 namespace {
@@ -1151,13 +1042,14 @@ void walk_tuned(const TraceArgs& A, int64_t n, int width, int tile, int stack, c
 }  // namespace
 
 cudaError_t launch_trace_dev(rt_scene_s* s, const rt_ray* rays, int64_t n, const int* n_dev, rt_hit* hits,
-                             uint8_t* occl, const rt_trace_params* tp, TraceScratch& scr, cudaStream_t st) {
+                             uint8_t* occl, const rt_trace_params* tp, cudaStream_t st) {
   cudaError_t e;
   int n_launched = 0;
   const bool quant = tp && (tp->flags & RT_QUANTIZED_NODES);
   if (quant && !s->q_built) return cudaErrorInvalidValue;  // no 64-byte nodes for this tree
   const int width = s->params.width == 8 ? 8 : 4;          // the traversal nodes the last build wrote
-  if ((e = cudaMemsetAsync(scr.counter, 0, 2 * sizeof(int), st))) return e;
+  int* const flagged = tp ? reinterpret_cast<int*>(tp->n_flagged_dev) : nullptr;
+  if (flagged && (e = cudaMemsetAsync(flagged, 0, sizeof(int), st))) return e;
   if (n > 0) {
     TraceArgs A;
     A.wide = s->wide;
@@ -1177,10 +1069,8 @@ cudaError_t launch_trace_dev(rt_scene_s* s, const rt_ray* rays, int64_t n, const
     A.skip = tp ? tp->skip_tri_dev : nullptr;
     const bool stats = tp && (tp->flags & RT_COUNT_STATS) && tp->stats_dev;
     A.stats = stats ? tp->stats_dev : nullptr;
-    A.counter = scr.counter;
-    A.queue = scr.queue;
-    A.cand = scr.cand;
-    A.qcap = (int)scr.cap;
+    A.counter = flagged;
+    A.retest = tp && (tp->flags & RT_NO_FP64_RETEST) ? 0 : 1;
     // ray tile (rays per CTA) and stack depth; the counting walk and the
     // 64-byte node walk use the defaults
     const int tile = (tp && !stats && !quant && (tp->block == 64 || tp->block == 256)) ? tp->block : kTraceBlock;
@@ -1203,27 +1093,6 @@ cudaError_t launch_trace_dev(rt_scene_s* s, const rt_ray* rays, int64_t n, const
       occl ? walk_tuned<true>(A, n, width, tile, stack, st) : walk_tuned<false>(A, n, width, tile, stack, st);
     }
     ++n_launched;
-    if (!(tp && (tp->flags & RT_NO_FP64_RETEST))) {
-      int g = (int)((n + kRetestBlock - 1) / kRetestBlock);
-      int gmax = sm_count_t() * 4;
-      g = g < gmax ? g : gmax;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)g);
-      cfg.blockDim = dim3(kRetestBlock);
-      cfg.stream = st;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      at[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      if ((e = occl ? cudaLaunchKernelEx(&cfg, k_retest64<true>, A) : cudaLaunchKernelEx(&cfg, k_retest64<false>, A)))
-        return e;
-      ++n_launched;
-    }
-  }
-  if (tp && tp->n_flagged_dev) {
-    if ((e = cudaMemcpyAsync(tp->n_flagged_dev, scr.counter, sizeof(int), cudaMemcpyDeviceToDevice, st)))
-      return e;
   }
   count_launches(n_launched);
   return cudaGetLastError();
@@ -1241,10 +1110,8 @@ cudaError_t launch_batch_persistent(rt_scene_s* s, const BatchLaunch& b, cudaStr
   A.root_ref = &s->ctl->root_ref;
   A.n_tri = (int)s->n_built;
   A.tris = s->tri_leaf;
-  A.counter = b.scr->counter;
-  A.queue = b.scr->queue;
-  A.cand = b.scr->cand;
-  A.qcap = (int)b.scr->cap;
+  A.counter = b.flagged;
+  A.retest = 1;
   A.n_dev = nullptr;
   A.stats = nullptr;
   P.tri_in = s->tri_in;
@@ -1273,7 +1140,7 @@ cudaError_t launch_batch_persistent(rt_scene_s* s, const BatchLaunch& b, cudaStr
   // zero; the flag counter too
   if ((e = cudaMemsetAsync(b.bar, 0, 4 * sizeof(unsigned), st))) return e;
   if ((e = cudaMemsetAsync(b.take, 0, (RT_BATCH_MAX_ORDER + 2) * sizeof(int), st))) return e;
-  if ((e = cudaMemsetAsync(b.scr->counter, 0, 2 * sizeof(int), st))) return e;
+  if ((e = cudaMemsetAsync(b.flagged, 0, sizeof(int), st))) return e;
   const bool w8 = s->params.width == 8;
   void (*k)(PersistArgs) = w8 ? k_batch<8> : k_batch<4>;
   static int per_sm[2] = {0, 0};
