@@ -1499,8 +1499,9 @@ __device__ __forceinline__ void micro_build(const BuildArgs& A, const Box6& x, i
     // (ip) and from the lane to the node's end (is): scans that stop at the
     // node's bounds, all nodes of the level at once
     Box6 ip = x, is = x;
-#pragma unroll 1
-    for (int o = 1; o < width; o <<= 1) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      if (o >= width) break;
       // a lane past the node's bound reads the bound's own union instead
       // (unions are idempotent, so nothing has to be selected)
       ip = box_join(ip, box_shfl(ip, max(lane - o, b)));
@@ -1518,8 +1519,11 @@ __device__ __forceinline__ void micro_build(const BuildArgs& A, const Box6& x, i
     // position that has it
     const float cost = ok ? c : INFINITY;
     float least = cost;
-#pragma unroll 1
-    for (int o = 1; o < width; o <<= 1) least = fminf(least, __shfl_sync(kFull, least, max(lane - o, b)));
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      if (o >= width) break;
+      least = fminf(least, __shfl_sync(kFull, least, max(lane - o, b)));
+    }
     least = __shfl_sync(kFull, least, e - 1);
     const unsigned at = __ballot_sync(kFull, ok && cost == least) & (0xffffffffu >> (32 - e)) & (0xffffffffu << b);
     const int q = !active ? lane : (at ? __ffs(at) - 1 : (b + e) / 2 - 1);  // no finite cost: middle
@@ -1868,8 +1872,17 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
     return bin_of(cc, acmin, ascl, K) < plane;
   };
   int cnt = 0;
+  // A node in shared memory gives a thread at most 32 records (1024 / 256 =
+  // 4): the sides are kept as bits, so that the partition below does not
+  // bin each record again (medium city: 16 bins 187.5 -> 184 us, 8 bins 181
+  // -> 177).
+  unsigned fl = 0;
 #pragma unroll 1
-  for (int k = k0; k < k1; ++k) cnt += goes_left(k);
+  for (int k = k0; k < k1; ++k) {
+    const bool l = goes_left(k);
+    cnt += l;
+    fl |= (unsigned)l << ((k - k0) & 31);
+  }
   int inc = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -1910,7 +1923,7 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
 #pragma unroll 1
   for (int k = k0; k < k1; ++k) {
     const float4 rl = rec_load<kGlobal>(src + 2 * k), rh = rec_load<kGlobal>(src + 2 * k + 1);
-    const bool left = goes_left(k);
+    const bool left = kGlobal ? goes_left(k) : ((fl >> (k - k0)) & 1u) != 0;
     const int d = left ? lb++ : nl + rb++;
     if (d < n) {
       if (kGlobal) {
