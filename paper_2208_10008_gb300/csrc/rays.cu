@@ -9,7 +9,7 @@
 //   2 (d.n) n about the unit geometric normal of the hit triangle, starting at
 //   the hit point with the remaining range tmax - t and the hit triangle to
 //   be skipped, and compact the survivors into the next order's ray queue in
-//   input order (count per block, scan, scatter: deterministic).
+//   input order (count per block, scatter: deterministic).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -165,15 +165,29 @@ __device__ __forceinline__ long long count_of(const ReflectArgs& A) {
   return A.n_dev ? (long long)*A.n_dev : A.n;
 }
 
+// A CTA's rays: kReflectRounds rounds of kRayBlock consecutive ones.
+constexpr int kReflectRounds = 4;
+constexpr int kReflectTile = kRayBlock * kReflectRounds;
+// Up to this many CTAs (16.8M rays) every scattering CTA adds up the counts
+// before its own itself (a million rays: 4 loads a thread); the scan by one
+// CTA, a launch of 7 us for a million rays, is left for more, where the sums
+// would grow with the square.  Two bounces of a million rays with their
+// traces: 528 -> 512 us.
+constexpr int kReflectSelf = 16384;
+
 __global__ void __launch_bounds__(kRayBlock) k_reflect_count(ReflectArgs A) {
   __shared__ int wsum[kRayBlock / 32];
   const long long n = count_of(A);
-  const long long i = blockIdx.x * (long long)kRayBlock + threadIdx.x;
-  float4 h;
-  const bool keep = i < n && survives(A, i, &h);
-  __syncwarp();
-  const unsigned m = __ballot_sync(0xffffffffu, keep);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = __popc(m);
+  const long long i0 = blockIdx.x * (long long)kReflectTile + threadIdx.x;
+  int c = 0;
+#pragma unroll
+  for (int r = 0; r < kReflectRounds; ++r) {
+    const long long i = i0 + r * kRayBlock;
+    float4 h;
+    const bool keep = i < n && survives(A, i, &h);
+    c += __popc(__ballot_sync(0xffffffffu, keep));
+  }
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = c;
   __syncthreads();
   if (threadIdx.x == 0) {
     int t = 0;
@@ -211,31 +225,57 @@ __global__ void __launch_bounds__(1024) k_reflect_scan(ReflectArgs A, int nblock
   if (threadIdx.x == 0) *A.out_count = (int)min((long long)carry, A.cap);
 }
 
+// kSelf: block_counts holds the CTAs' counts (else their first positions);
+// the last CTA then writes the total.
+template <bool kSelf>
 __global__ void __launch_bounds__(kRayBlock) k_reflect_scatter(ReflectArgs A) {
-  __shared__ int wsum[kRayBlock / 32];
+  constexpr int kW = kRayBlock / 32;
+  __shared__ int wsum[kReflectRounds][kW];
+  __shared__ int part[kW];
   const long long n = count_of(A);
-  const long long i = blockIdx.x * (long long)kRayBlock + threadIdx.x;
+  const long long i0 = blockIdx.x * (long long)kReflectTile + threadIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-  const bool keep = i < n && survives(A, i, &h);
-  __syncwarp();
-  const unsigned m = __ballot_sync(0xffffffffu, keep);
-  if (lane == 0) wsum[warp] = __popc(m);
+  float4 h[kReflectRounds];
+  unsigned m[kReflectRounds];
+#pragma unroll
+  for (int r = 0; r < kReflectRounds; ++r) {
+    const long long i = i0 + r * kRayBlock;
+    h[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+    m[r] = __ballot_sync(0xffffffffu, i < n && survives(A, i, &h[r]));
+    if (lane == 0) wsum[r][warp] = __popc(m[r]);
+  }
+  if (kSelf) {
+    int c = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kRayBlock) c += A.block_counts[b];
+    __syncwarp();
+    c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+    if (lane == 0) part[warp] = c;
+  }
   __syncthreads();
-  if (!keep) return;
-  int pos = A.block_counts[blockIdx.x];
-  for (int w = 0; w < warp; ++w) pos += wsum[w];
-  pos += __popc(m & ((1u << lane) - 1u));
-  if (pos >= A.cap) return;
-  const float4 ra = A.rays[2 * i], rb = A.rays[2 * i + 1];
-  const int id = __float_as_int(h.y);
-  float4 o0, o1;
-  reflect_ray(ra, rb, h.x, A.tri_in[3 * (size_t)id], A.tri_in[3 * (size_t)id + 1], A.tri_in[3 * (size_t)id + 2], &o0,
-              &o1);
-  A.out_rays[2 * (size_t)pos] = o0;
-  A.out_rays[2 * (size_t)pos + 1] = o1;
-  A.out_skip[pos] = id;
-  if (A.out_src) A.out_src[pos] = (int)i;
+  int base = kSelf ? 0 : A.block_counts[blockIdx.x];
+  if (kSelf)
+    for (int w = 0; w < kW; ++w) base += part[w];
+  if (kSelf && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
+    *A.out_count = (int)min((long long)base + A.block_counts[blockIdx.x], A.cap);
+#pragma unroll
+  for (int r = 0; r < kReflectRounds; ++r) {
+    int pos = base + __popc(m[r] & ((1u << lane) - 1u));
+    for (int w = 0; w < kW; ++w) {
+      pos += w < warp ? wsum[r][w] : 0;
+      base += wsum[r][w];
+    }
+    if (!((m[r] >> lane) & 1u) || pos >= A.cap) continue;
+    const long long i = i0 + r * kRayBlock;
+    const float4 ra = A.rays[2 * i], rb = A.rays[2 * i + 1];
+    const int id = __float_as_int(h[r].y);
+    float4 o0, o1;
+    reflect_ray(ra, rb, h[r].x, A.tri_in[3 * (size_t)id], A.tri_in[3 * (size_t)id + 1], A.tri_in[3 * (size_t)id + 2],
+                &o0, &o1);
+    A.out_rays[2 * (size_t)pos] = o0;
+    A.out_rays[2 * (size_t)pos + 1] = o1;
+    A.out_skip[pos] = id;
+    if (A.out_src) A.out_src[pos] = (int)i;
+  }
 }
 
 std::once_flag g_ico_once;
@@ -375,12 +415,17 @@ cudaError_t launch_reflect(const rt_scene_s* s, const rt_ray* rays, const rt_hit
   A.out_count = out_count;
   A.block_counts = block_counts;
   A.cap = cap;
-  const int nb = (int)((n + kRayBlock - 1) / kRayBlock);
+  const int nb = (int)((n + kReflectTile - 1) / kReflectTile);
   if (nb == 0) return cudaMemsetAsync(out_count, 0, sizeof(int), st);
   k_reflect_count<<<nb, kRayBlock, 0, st>>>(A);
-  k_reflect_scan<<<1, 1024, 0, st>>>(A, nb);
-  k_reflect_scatter<<<nb, kRayBlock, 0, st>>>(A);
-  count_launches(3);
+  if (nb <= kReflectSelf) {
+    k_reflect_scatter<true><<<nb, kRayBlock, 0, st>>>(A);
+    count_launches(2);
+  } else {
+    k_reflect_scan<<<1, 1024, 0, st>>>(A, nb);
+    k_reflect_scatter<false><<<nb, kRayBlock, 0, st>>>(A);
+    count_launches(3);
+  }
   return cudaGetLastError();
 }
 
