@@ -692,7 +692,8 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         }
         continue;
       }
-      // certain hit: near an end of the interval the float64 rule decides
+      // certain hit: near an end of the interval the float64 rule decides; it
+      // may turn the hit down, so such a hit must not cull what lies behind it
       const bool near_end = fabsf(h.t - r.tmax) <= h.err + kTieRel * fabsf(r.tmax) ||
                             fabsf(h.t - r.tmin) <= h.err + kTieRel * fabsf(h.t);
       if (near_end) flag = true;
@@ -721,12 +722,12 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         t2 = h.t;
         e2 = h.err;
       }
-      bound = fminf(r.tmax, t1 + kTieRel * t1 + e1);
+      if (!near_end) bound = fminf(bound, h.t + kTieRel * fabsf(h.t) + h.err);
     }
   }
   if (kAny) {
     if (done) flag = false;
-  } else if (t2 < INFINITY && t2 <= t1 + kTieRel * t1 + e1 + e2) {
+  } else if (t2 < INFINITY && t2 <= t1 + kTieRel * fabsf(t1) + e1 + e2) {
     flag = true;
   }
   if (A.counter) {
