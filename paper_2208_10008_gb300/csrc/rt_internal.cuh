@@ -196,8 +196,9 @@ struct BuildGeom {
 };
 BuildGeom build_geometry(int64_t n_tri, int nsm);
 
-// Float64 candidates that a walk remembers per ray.
-constexpr int kTraceCand = 8;
+// Float64 candidates that a walk remembers per ray (16, 24 and 32: a launch of
+// which 10% aim at the tips of 48-sided cones 5.19, 4.45 and 5.08 ms).
+constexpr int kTraceCand = 24;
 
 // Order-preserving float <-> int map for atomicMin/atomicMax on floats.
 __host__ __device__ inline int ford(float f) {

@@ -23,12 +23,12 @@
 //     functions.  Signs settled beyond E give a certain hit or miss; anything
 //     else, a second hit within the error window of the best one, a hit near
 //     tmin / tmax, or a stack overflow marks the ray for the float64 pass.
-// retest_ray (float64, flagged rays only, at the end of their walk)
+// retest_warp (float64, flagged rays only, at the end of their warp's walk)
 //   * applies the float64 rule to the candidates the walk remembered and keeps
-//     the nearest; when the list overflowed, a stackless walk of the
-//     binary tree (parent links) with the same conservative float32 box test
-//     culled at the float64 best distance, and for every triangle the
-//     float32 bound does not prove missed, the reference hit rule:
+//     the nearest; when the list or the stack was too short, a stackless walk
+//     of the binary tree (parent links) with the same conservative float32 box
+//     test, culled at the walk's bound and the float64 best distance, collects
+//     every triangle the float32 bound does not prove missed.  The rule:
 //     Moller-Trumbore with inclusive edges, |det| <= 1e-14 |e1||e2||d| is
 //     parallel, tmin < t < tmax, lowest id on equal t, with the operation
 //     order fixed and no contraction, so its answer is the float64
@@ -425,116 +425,196 @@ __device__ bool mt64(D3 o, D3 d, D3 v0, D3 v1, D3 v2, double* t, double* u, doub
   return true;
 }
 
-// The float64 pass of ray i, which the float32 walk flagged: its candidates
-// (leaf positions cand[0 .. nc)) by the float64 rule, the nearest kept, the
-// lowest id on ties; without a complete list (nc < 0) every triangle that the
-// float32 bound does not prove missed.  Called by the flagged lanes at the
-// end of their walk, a few dozen of 655,362 on the medium city, while other
-// warps walk: as a kernel of its own behind the walk (queue, counter, a group
-// of lanes per ray) it took 12 us of the 110 us of a trace, most of them its
-// launch and its chain of dependent loads and float64 operations.  Not
-// inlined, so that the walk's registers are its own.
-template <bool kAny>
-__device__ __noinline__ void retest_ray(const TraceArgs& A, const float4* r4, const int skip, const int* cand,
-                                        const int nc, float4* hit, uint8_t* occl) {
-  const float4 ra = r4[0], rb = r4[1];
+// The float64 answer of a ray so far: the nearest hit, the lowest id on ties.
+struct Best64 {
+  double t, u, v;
+  int id, pos;  // id INT_MAX: none
+};
+__device__ __forceinline__ Best64 best64_none() { return {INFINITY, 0.0, 0.0, INT_MAX, -1}; }
+
+// The float64 rule for ray (ra, rb) and the triangle (va, vb, vc) at leaf position pos.
+__device__ __forceinline__ Best64 hit64(float4 ra, float4 rb, float4 va, float4 vb, float4 vc, int pos) {
+  Best64 h = best64_none();
+  double t, u, v;
+  if (mt64(D3{ra.x, ra.y, ra.z}, D3{rb.x, rb.y, rb.z}, D3{va.x, va.y, va.z}, D3{vb.x, vb.y, vb.z},
+           D3{vc.x, vc.y, vc.z}, &t, &u, &v) &&
+      t > (double)ra.w && t < (double)rb.w)
+    h = {t, u, v, __float_as_int(va.w), pos};
+  return h;
+}
+__device__ __forceinline__ bool nearer64(double t, int id, double t0, int id0) {
+  return t < t0 || (t == t0 && id < id0);
+}
+
+// The hit record of a ray settled in float64.  The record is a function of
+// the ray and the winning triangle only: where the float32 test certifies the
+// winner, report exactly what the float32 walk reports for it (so the result
+// never depends on whether this tree's walk flagged the ray).
+__device__ __forceinline__ float4 record64(const float4* tris, float4 ra, float4 rb, const Best64& w) {
+  if (w.id == INT_MAX) return make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
   const RayPre r = setup_ray(ra, rb);
-  const D3 o{ra.x, ra.y, ra.z}, d{rb.x, rb.y, rb.z};
-  const double tmin = ra.w, tmax = rb.w;
-  double bt = INFINITY, bu = 0.0, bv = 0.0;
-  int bid = -1, bpos = -1;
-  bool any = false;
-  auto test = [&](int pos, float4 va, float4 vb, float4 vc) {
-    double t, u, v;
-    if (mt64(o, d, D3{va.x, va.y, va.z}, D3{vb.x, vb.y, vb.z}, D3{vc.x, vc.y, vc.z}, &t, &u, &v) && t > tmin &&
-        t < tmax) {
-      any = true;
-      const int id = __float_as_int(va.w);
-      if (t < bt || (t == bt && (bid < 0 || id < bid))) {
-        bt = t;
-        bid = id;
-        bpos = pos;
-        bu = u;
-        bv = v;
-      }
+  const float4* tp = tris + 3 * (size_t)w.pos;
+  const float4 va = tp[0], vb = tp[1], vc = tp[2];
+  const TriRes h = tri_test(r, va, vb, vc);
+  if (h.cls == 1 && h.t > r.tmin && h.t < r.tmax) {
+    float t = h.t;
+    if (h.err > 0.25f * (kTieRel * h.t + 1e-6f)) t = refine_t(r, rb.x, rb.y, rb.z, va, vb, vc);
+    return make_float4(t, __int_as_float(w.id), h.u, h.v);
+  }
+  return make_float4((float)w.t, __int_as_float(w.id), (float)w.u, (float)w.v);
+}
+
+// Where a ray's second walk, through the binary tree, has come to.
+struct TreeWalk {
+  int node, s;  // s: next child of `node` to try (2: done); node INT_MIN: not begun
+  long long steps;
+};
+
+// Collects the triangles that the float32 bound does not prove missed into
+// cand, from where w stands, in the boxes nearer than bound: a stackless walk
+// of the binary tree (parent links), so that any depth works, with the walk's
+// own widened slab test.  Returns their number; stops when the next leaf might
+// not fit, and sets *more to false at the end of the tree.  (A cull of the
+// triangles by their distance too takes registers from the walk around it:
+// 1,000,003 segments 508 -> 517 us, a launch of 262,143 random rays 238 -> 244.)
+static_assert(kCand >= kMaxLeaf, "an empty list holds a leaf");
+__device__ __noinline__ int walk_tree(const TraceArgs& A, const float4* r4, const int skip, float bound, TreeWalk* w,
+                                      int* cand, bool* more) {
+  const RayPre r = setup_ray(r4[0], r4[1]);
+  bound = bound + fabsf(bound) * 2e-6f;
+  int nc = 0;
+  auto leaf = [&](int ref) {
+    const int first = leaf_first(ref), count = leaf_count(ref);
+    for (int k = 0; k < count; ++k) {
+      const float4* tp = A.tris + 3 * (size_t)(first + k);
+      const float4 va = tp[0], vb = tp[1], vc = tp[2];
+      if (__float_as_int(va.w) != skip && tri_test(r, va, vb, vc).cls != 0) cand[nc++] = first + k;
     }
   };
+  const int root = *A.root_ref;
+  *more = false;
+  if (!r.valid || root >= A.n_tri - 1) return 0;  // (the latter: no usable tree)
+  if (root < 0) {
+    if (root != INT_MIN) leaf(root);
+    return nc;
+  }
+  int node = w->node == INT_MIN ? root : w->node, s = w->s;
+  long long steps = w->steps;
+  for (; steps < (1ll << 32); ++steps) {
+    if (nc > kCand - kMaxLeaf) {
+      *w = {node, s, steps};
+      *more = true;
+      break;
+    }
+    if (s < 2) {
+      const Node2* nd = A.node2 + node;
+      const float4 lo = s == 0 ? nd->a_lo : nd->b_lo, hi = s == 0 ? nd->a_hi : nd->b_hi;
+      ++s;
+      if (!slab1(lo, hi, r, bound)) continue;
+      const int ref = __float_as_int(lo.w);
+      if (ref < 0) {
+        leaf(ref);
+      } else if (ref < A.n_tri - 1) {  // (a link the build never wrote is skipped)
+        node = ref;
+        s = 0;
+      }
+      continue;
+    }
+    if (node == root) break;
+    const int p = A.link2[node].x;
+    if (p < 0 || p >= A.n_tri - 1) break;
+    s = __float_as_int(A.node2[p].a_lo.w) == node ? 1 : 2;
+    node = p;
+  }
+  return nc;
+}
+
+// The float64 pass of a warp's rays, at the end of their walk, while other
+// warps walk.  Each lane brings the nc candidates of its ray i (leaf positions
+// cand[0 .. nc); nc < 0: its ray is settled); the candidates of all lanes are
+// dealt out to the 32 lanes, so that a warp with two flagged rays of ten
+// candidates each runs the float64 rule once and not ten times: float64 is
+// what the device has least of, a warp's instruction occupies the SM for 16
+// cycles whatever its lanes.  Rays without a complete list (more) then collect
+// theirs, a list at a time, from the boxes nearer than bound, where the walk
+// has proved a hit, or the float64 best.  Called by whole warps; not inlined,
+// so that the walk's registers are its own.
+//
+// 1,048,576 launched rays on the medium city, a share of them aimed at
+// vertices: each lane on its own, with a walk of the whole tree for more than
+// 8 candidates, 196 us at 0.01%, 972 at 5%, 1520 at 10% and 3720 at 50%; now
+// 126, 320, 426 and 819 (none: 124 and 120).  A queue and a kernel of its own
+// for the flagged rays: 253, 756, 1012 and 3030.
+template <bool kAny>
+__device__ __noinline__ void retest_warp(const TraceArgs& A, const rt_ray* rays, const int i, const int skip,
+                                         int* cand, int nc, bool more, const float bound, rt_hit* hits,
+                                         uint8_t* occl) {
+  const int lane = threadIdx.x & 31;
+  const float4* r4 = reinterpret_cast<const float4*>(rays);
+  const bool own = nc >= 0;
+  TreeWalk w{INT_MIN, 0, 0};
+  Best64 best = best64_none();
 #pragma unroll 1
-  for (int q = 0; q < nc; ++q) {
-    const float4* tp = A.tris + 3 * (size_t)cand[q];
-    const float4 va = tp[0];
-    if (__float_as_int(va.w) != skip) test(cand[q], va, tp[1], tp[2]);
-  }
-  if (nc < 0 && r.valid) {
-    // A stackless walk of the binary tree (parent links), so that any depth
-    // works.  Boxes use the same widened float32 slab test as the walk, culled
-    // at the float64 best distance rounded up.
-    auto test_leaf = [&](int ref) {
-      const int first = leaf_first(ref), count = leaf_count(ref);
-      for (int k = 0; k < count && !(kAny && any); ++k) {
-        const float4* tp = A.tris + 3 * (size_t)(first + k);
-        const float4 va = tp[0], vb = tp[1], vc = tp[2];
-        if (__float_as_int(va.w) == skip) continue;
-        if (tri_test(r, va, vb, vc).cls == 0) continue;  // certain miss
-        test(first + k, va, vb, vc);
-      }
-    };
-    const int root = *A.root_ref;
-    if (root >= A.n_tri - 1) {
-      // no usable tree: nothing to walk
-    } else if (root < 0) {
-      if (root != INT_MIN) test_leaf(root);
-    } else {
-      int node = root, s = 0;  // s: next child of `node` to try (2: done)
-      for (long long guard = 0; guard < (1ll << 32); ++guard) {
-        if (s < 2) {
-          const Node2* nd = A.node2 + node;
-          const float4 lo = s == 0 ? nd->a_lo : nd->b_lo, hi = s == 0 ? nd->a_hi : nd->b_hi;
-          float bf = (float)fmin(bt, tmax);
-          bf = bf + fabsf(bf) * 2e-6f;
-          ++s;
-          if (!slab1(lo, hi, r, bf)) continue;
-          const int ref = __float_as_int(lo.w);
-          if (ref >= 0) {
-            if (ref < A.n_tri - 1) {  // a link the build never wrote is skipped
-              node = ref;
-              s = 0;
-            }
-            continue;
-          }
-          test_leaf(ref);
-          if (kAny && any) break;
-          continue;
-        }
-        if (node == root) break;
-        const int p = A.link2[node].x;
-        if (p < 0 || p >= A.n_tri - 1) break;
-        s = __float_as_int(A.node2[p].a_lo.w) == node ? 1 : 2;
-        node = p;
-      }
+  for (;;) {
+    __syncwarp();
+    const int c = max(nc, 0);
+    int x = c;  // candidates of the lanes up to this one
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFullMask, x, o);
+      x += lane >= o ? y : 0;
     }
-  }
-  if (kAny) {
-    *occl = any ? 1 : 0;
-    return;
-  }
-  float4 out = make_float4(INFINITY, __int_as_float(-1), 0.f, 0.f);
-  if (bid >= 0) {
-    out = make_float4((float)bt, __int_as_float(bid), (float)bu, (float)bv);
-    // The record is a function of the ray and the winning triangle only:
-    // where the float32 test certifies the winner, report exactly what
-    // the float32 walk reports for it (so the result never depends on
-    // whether this tree's walk flagged the ray).
-    const float4* tp = A.tris + 3 * (size_t)bpos;
-    const float4 va = tp[0], vb = tp[1], vc = tp[2];
-    const TriRes h = tri_test(r, va, vb, vc);
-    if (h.cls == 1 && h.t > r.tmin && h.t < r.tmax) {
-      float t = h.t;
-      if (h.err > 0.25f * (kTieRel * h.t + 1e-6f)) t = refine_t(r, rb.x, rb.y, rb.z, va, vb, vc);
-      out = make_float4(t, __int_as_float(bid), h.u, h.v);
+    const int total = __shfl_sync(kFullMask, x, 31);
+    const int most = (int)__reduce_max_sync(kFullMask, (unsigned)c);
+#pragma unroll 1
+    for (int t0 = 0; t0 < total; t0 += 32) {
+      const int task = min(t0 + lane, total - 1);  // (past the end the last one again: the least of equals is itself)
+      int f = 0;                                   // the task's lane: the first with more than `task` up to it
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) f += __shfl_sync(kFullMask, x, f + o - 1) <= task ? o : 0;
+      const int q = task - (__shfl_sync(kFullMask, x, f) - __shfl_sync(kFullMask, c, f));
+      int pos = 0;
+#pragma unroll 1
+      for (int k = 0; k < most; ++k) {
+        const int p = __shfl_sync(kFullMask, k < c ? cand[k] : 0, f);
+        pos = k == q ? p : pos;
+      }
+      const size_t ri = 2 * (size_t)__shfl_sync(kFullMask, i, f);
+      const float4* tp = A.tris + 3 * (size_t)pos;
+      const Best64 h = hit64(r4[ri], r4[ri + 1], tp[0], tp[1], tp[2], pos);
+      // the nearest of each ray's run of lanes, at the run's first lane
+      double t = h.t;
+      int id = h.id, at = lane;
+      __syncwarp();
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int from = min(lane + o, 31);
+        const double t2 = __shfl_sync(kFullMask, t, from);
+        const int id2 = __shfl_sync(kFullMask, id, from), at2 = __shfl_sync(kFullMask, at, from);
+        const bool take = __shfl_sync(kFullMask, f, from) == f && nearer64(t2, id2, t, id);
+        t = take ? t2 : t;
+        id = take ? id2 : id;
+        at = take ? at2 : at;
+      }
+      const bool mine = c > 0 && x > t0 && x - c < t0 + 32;  // this round holds candidates of the lane's own ray
+      const int src = mine ? max(x - c - t0, 0) : lane;
+      t = __shfl_sync(kFullMask, t, src);
+      id = __shfl_sync(kFullMask, id, src);
+      at = __shfl_sync(kFullMask, at, src);
+      const double u = __shfl_sync(kFullMask, h.u, at), v = __shfl_sync(kFullMask, h.v, at);
+      pos = __shfl_sync(kFullMask, h.pos, at);
+      if (mine && nearer64(t, id, best.t, best.id)) best = {t, u, v, id, pos};
     }
+    more = more && !(kAny && best.id != INT_MAX);
+    if (!__any_sync(kFullMask, more)) break;
+    nc = 0;
+    if (more) nc = walk_tree(A, r4 + 2 * (size_t)i, skip, (float)fmin(best.t, (double)bound), &w, cand, &more);
   }
-  *hit = out;
+  if (!own) return;
+  if (kAny)
+    occl[i] = best.id != INT_MAX ? 1 : 0;
+  else
+    reinterpret_cast<float4*>(hits)[i] = record64(A.tris, r4[2 * (size_t)i], r4[2 * (size_t)i + 1], best);
 }
 
 // ---------------------------------------------------------------- the walk
@@ -565,7 +645,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
   int cpos[kCand];
   float clo[kCand];
   int nc = 0;
-  bool walk_all = false;
+  bool walk_all = false;  // the list or the stack was too short
   auto remember = [&](int pos, float lo) {
     if (nc == kCand) {  // make room: drop entries already beyond the cull bound
       int w = 0;
@@ -607,13 +687,12 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         float tn[8];
         int ch[8];
         const unsigned m = slab8(A.wide8 + ref, r, bound, tn, ch);
-        const int cnt = __popc(m);
+        int cnt = __popc(m);
         if (cnt == 0) continue;
-        if (sp + cnt - 1 > kSD) {  // cannot hold the children: leave it to the float64 pass
+        if (sp + cnt - 1 > kSD) {  // cannot hold the farthest: the float64 pass finds what is in them
           flag = true;
           walk_all = true;
-          sp = 0;
-          continue;
+          cnt = kSD + 1 - sp;
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
@@ -659,11 +738,10 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       cswap(tb, rb, tc, rc);
       int cnt = __popc(m);
       if (cnt == 0) continue;
-      if (sp + cnt - 1 > kSD) {  // cannot hold the children: leave it to the float64 pass
+      if (sp + cnt - 1 > kSD) {  // cannot hold the farthest: the float64 pass finds what is in them
         flag = true;
         walk_all = true;
-        sp = 0;
-        continue;
+        cnt = kSD + 1 - sp;
       }
       // push farthest first so the nearest stacked one is popped next
       if (cnt > 3) st[sp++] = make_int2(rd, __float_as_int(td));
@@ -730,22 +808,23 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
   } else if (t2 < INFINITY && t2 <= t1 + kTieRel * fabsf(t1) + e1 + e2) {
     flag = true;
   }
-  if (A.counter) {
-    const unsigned m = __ballot_sync(kFullMask, flag);
-    if ((threadIdx.x & 31) == 0 && m) atomicAdd(A.counter, __popc(m));
+  const unsigned flagged = __ballot_sync(kFullMask, flag);
+  if (A.counter && flagged && (threadIdx.x & 31) == 0) atomicAdd(A.counter, __popc(flagged));
+  if (flagged && A.retest) {
+    int w = -1;
+    if (flag) {
+      w = 0;
+      for (int q = 0; q < nc; ++q)
+        if (clo[q] <= bound) cpos[w++] = cpos[q];
+    }
+    retest_warp<kAny>(A, rays, i, skip, cpos, w, flag && walk_all, bound, hits, occl);
   }
   if (!live) return;
   if (kStats && A.stats) {
     A.stats[2 * (size_t)i] = n_nodes;
     A.stats[2 * (size_t)i + 1] = n_tris;
   }
-  if (flag && A.retest) {
-    int w = 0;
-    for (int q = 0; q < nc; ++q)
-      if (clo[q] <= bound) cpos[w++] = cpos[q];
-    retest_ray<kAny>(A, r4, skip, cpos, walk_all ? -1 : w, reinterpret_cast<float4*>(hits) + i, occl + i);
-    return;
-  }
+  if (flag && A.retest) return;
   if (kAny) {
     occl[i] = done ? 1 : 0;
   } else {
