@@ -622,16 +622,18 @@ __device__ __noinline__ void retest_warp(const TraceArgs& A, const rt_ray* rays,
 // statistics and the flag for the float64 pass.  Called by whole warps;
 // lanes without a ray pass live = false.  A lane visits the same boxes and
 // triangles in the same order whatever its warp does, so its result does not
-// depend on the other lanes.
-template <bool kAny, bool kStats, int kSD, bool kQuant, int kW>
+// depend on the other lanes.  kWritten: the rays and skips were written by this
+// launch (a batch's bounced orders), which read-only loads must not be used on.
+template <bool kAny, bool kStats, int kSD, bool kQuant, int kW, bool kWritten>
 __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const bool live,
                                          const rt_ray* __restrict__ rays,
                                          rt_hit* __restrict__ hits, uint8_t* __restrict__ occl,
                                          const int32_t* __restrict__ skip_ids) {
   const float4* r4 = reinterpret_cast<const float4*>(rays) + 2 * (size_t)i;
   const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);  // (an invalid ray: no direction)
-  const RayPre r = setup_ray(live ? __ldg(r4) : none, live ? __ldg(r4 + 1) : none);
-  const int skip = live && skip_ids ? __ldg(skip_ids + i) : -1;
+  auto load = [](const auto* p) { return kWritten ? __ldcg(p) : __ldg(p); };
+  const RayPre r = setup_ray(live ? load(r4) : none, live ? load(r4 + 1) : none);
+  const int skip = live && skip_ids ? load(skip_ids + i) : -1;
   float t1 = INFINITY, t2 = INFINITY, e1 = 0.f, e2 = 0.f, bu = 0.f, bv = 0.f;
   int id1 = -1, pos1 = -1;
   bool flag = false, done = false;
@@ -831,7 +833,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
     if (id1 >= 0 && e1 > 0.25f * (kTieRel * t1 + 1e-6f)) {
       // the float32 distance is not certified inside the tolerance: recompute it
       const float4* tp = A.tris + 3 * (size_t)pos1;
-      const float4 rb4 = __ldg(r4 + 1);
+      const float4 rb4 = load(r4 + 1);
       t1 = refine_t(r, rb4.x, rb4.y, rb4.z, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
     }
     float4 out = id1 >= 0 ? make_float4(t1, __int_as_float(id1), bu, bv)
@@ -854,7 +856,7 @@ template <bool kAny, bool kStats, int kTile, int kSD, bool kQuant, int kW = 4>
 __global__ void __launch_bounds__(kTile, walk_ctas<kAny, kStats, kTile, kSD, kQuant, kW>()) k_trace(TraceArgs A) {
   const int i = blockIdx.x * kTile + threadIdx.x;
   const bool live = i < A.n && !(A.n_dev && i >= *A.n_dev);
-  walk_one<kAny, kStats, kSD, kQuant, kW>(A, i, live, A.rays, A.hits, A.occl, A.skip);
+  walk_one<kAny, kStats, kSD, kQuant, kW, false>(A, i, live, A.rays, A.hits, A.occl, A.skip);
 }
 
 // ---------------------------------------------------------------- one launch for a whole batch
@@ -955,7 +957,7 @@ __device__ __forceinline__ void walk_phase(const TraceArgs& A, int* take, int n,
     if (lane == 0) b = atomicAdd(take, 32);
     b = __shfl_sync(kFullMask, b, 0);
     if (b >= n) break;
-    walk_one<kAny, false, kStack, false, kW>(A, b + lane, b + lane < n, rays, hits, occl, skip);
+    walk_one<kAny, false, kStack, false, kW, true>(A, b + lane, b + lane < n, rays, hits, occl, skip);
   }
 }
 
