@@ -524,9 +524,9 @@ typedef struct {
  * and max_slots concurrent requests (1..64), each on its own stream.  A
  * worker thread admits queued requests in arrival order whenever a slot is
  * free and the pool holds all of the request's buffers (rays, hits, skip and
- * parent arrays per order, and 44 bytes a ray that are not used any more:
- * about n * (56 (max_order + 1) + 44) bytes for n rays), so requests of uneven sizes run side by side on the
- * device.  The calling thread's current device is used.
+ * parent arrays per order: about 56 n (max_order + 1) bytes for n rays), so
+ * requests of uneven sizes run side by side on the device.  The calling
+ * thread's current device is used.
  * Errors: RT_EINVAL, RT_ENOMEM, RT_ECUDA. */
 int rt_session_create(size_t pool_bytes, int max_slots, rt_session* out);
 

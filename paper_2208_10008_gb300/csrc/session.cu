@@ -192,7 +192,6 @@ size_t request_bytes(long long n, int orders) {
   size_t b = per_order * (size_t)(orders + 1);
   b += 64 + (size_t)(RT_BATCH_MAX_ORDER + 1) * sizeof(int);      // counts
   b += ((size_t)n / 256 + 2) * sizeof(int);                       // reflect blocks
-  b += 64 + (size_t)n * sizeof(int) * 10;                         // not used: a request's size decides which are refused
   return b + 64 * 256;                                            // alignment slack (<= 48 arrays)
 }
 
