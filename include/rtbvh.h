@@ -165,9 +165,10 @@ int rt_bvh_build(rt_scene scene, const rt_build_params* params, void* stream);
 
 /* Instrumentation, with no counterpart in the paper: record the CUDA events
  * ev_begin and ev_end (cudaEvent_t passed as void*) on the build stream just
- * before and just after the split kernel (the recursion of Fig. 2, the
- * build's longest kernel) of every later rt_bvh_build of this scene, so
- * that the caller can time that kernel alone (cudaEventElapsedTime).  Both
+ * before and just after the kernels that split nodes (the recursion of
+ * Fig. 2: one kernel, or two from 240,000 triangles, which leave the small
+ * subtrees to the second) of every later rt_bvh_build of this scene, so that
+ * the caller can time the recursion alone (cudaEventElapsedTime).  Both
  * NULL stops it.  Inside a stream capture the records become event-record
  * nodes of the graph.  The events stay the caller's and must outlive the
  * builds that record them.  Errors: RT_EINVAL (scene NULL, or only one of

@@ -2853,11 +2853,11 @@ cudaError_t launch_build(rt_scene_s* s, const rt_build_params& p, cudaStream_t s
   if (s->split_ev[0] && (e = cudaEventRecordWithFlags(s->split_ev[0], st, evflags))) return e;
   if ((e = launch(large ? k_split<true> : k_split<false>, split_per_sm * nsm, split_smem(large), st, true, A)))
     return e;
-  if (s->split_ev[1] && (e = cudaEventRecordWithFlags(s->split_ev[1], st, evflags))) return e;
   if (A.wsm) {
     if ((e = launch(k_small, 3 * nsm, 0, st, true, A))) return e;
     count_launches(1);
   }
+  if (s->split_ev[1] && (e = cudaEventRecordWithFlags(s->split_ev[1], st, evflags))) return e;
   if ((e = launch(k_post, gp, 0, st, true, A))) return e;
   count_launches(4);
   return cudaSuccess;

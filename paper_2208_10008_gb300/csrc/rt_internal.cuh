@@ -425,7 +425,7 @@ struct rt_scene_s {
   cudaStream_t host_streams[2] = {nullptr, nullptr};
   cudaEvent_t host_ev = nullptr;  // the host pipeline's wait on the caller's stream
   cudaEvent_t ev_build0 = nullptr, ev_build1 = nullptr;
-  cudaEvent_t split_ev[2] = {nullptr, nullptr};  // caller's events around the split kernel
+  cudaEvent_t split_ev[2] = {nullptr, nullptr};  // caller's events around the split kernels
   bool built = false;
   rt_build_params params{};
   // range-limited builds: the selected triangles' ids, per-block counts, the

@@ -297,8 +297,8 @@ def rt_bvh_build(scene: Scene, stream=None, **kw):
 
 
 def rt_scene_set_split_events(scene: Scene, ev_begin=None, ev_end=None):
-    """Record two torch.cuda.Event (timing enabled) around the split kernel of
-    every later build of `scene`; no arguments stops it."""
+    """Record two torch.cuda.Event (timing enabled) around the split kernels (the
+    whole recursion) of every later build of `scene`; no arguments stops it."""
     for e in (ev_begin, ev_end):
         if e is not None and not e.cuda_event:
             e.record()  # torch creates its event on the first record
