@@ -58,7 +58,7 @@ constexpr int kBinWords = 3 * kMaxBins * kBinVals;
 constexpr int kCntStride = 3 * kMaxBins;
 constexpr int kMaxRpt = 8;     // records per thread of a big node's chunk
 constexpr int kRegRpt = 4;     // at most, where they stay in registers
-constexpr int kStage = 2048;   // of a chunk's records in shared memory at a time
+constexpr int kStage = kBlock * kMaxRpt;  // records of a chunk in shared memory: all of them
 constexpr int kLargeScene = 240000;  // records from which a build is bound by work and not by its longest chain
 constexpr int kBigMin = 1024;  // big nodes have more triangles than this
 constexpr unsigned kFull = 0xffffffffu;
@@ -842,7 +842,7 @@ __device__ __forceinline__ void note_node(WarpStats& ws, int nl, int nr, bool le
 }
 
 // ------------------------------------------------------------------ big nodes
-// Shared-memory place of record k of a stage, in float4: four records and
+// Shared-memory place of record k of a chunk, in float4: four records and
 // 16 bytes of padding per thread, so that 16-byte reads of consecutive
 // records by consecutive lanes fall on distinct banks.
 __device__ __forceinline__ int stage_at(int k) { return (k >> 2) * 9 + (k & 3) * 2; }
@@ -862,7 +862,7 @@ struct TopSmem {
   int np;
 };
 
-// With a stage of the chunk's records.
+// With the chunk's records.
 struct StagedSmem {
   TopSmem top;
   alignas(16) float4 rec[kStage / 4 * 9];  // (stage_at)
@@ -981,22 +981,14 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   float4* dst = A.rec[par ^ 1];
   const int r0 = j * CH;
   const int rn = min(CH, n - r0);
-  // the chunk's records go to shared memory stage by stage, the first while
-  // the split is chosen
-  auto fetch = [&](int g) {
-    const int m = min(kStage, rn - g * kStage);
-    if (m > 0) {
-      const float4* p = src + 2 * ((size_t)T.begin + r0 + g * kStage);
-      const unsigned to = (unsigned)__cvta_generic_to_shared(&G.rec[0]);
-      for (int i = tid; i < 2 * m; i += kBlock)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * (stage_at(i >> 1) + (i & 1))),
-                     "l"(p + i)
-                     : "memory");
-    }
-  };
   float4 lo[kRegRpt], hi[kRegRpt];
-  if (kStaged) {
-    fetch(0);
+  if (kStaged) {  // the chunk's records go to shared memory while the split is chosen
+    const float4* p = src + 2 * ((size_t)T.begin + r0);
+    const unsigned to = (unsigned)__cvta_generic_to_shared(&G.rec[0]);
+    for (int i = tid; i < 2 * rn; i += kBlock)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * (stage_at(i >> 1) + (i & 1))),
+                   "l"(p + i)
+                   : "memory");
   } else {
 #pragma unroll
     for (int r = 0; r < kRegRpt; ++r) {
@@ -1110,18 +1102,16 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
   const int dnext0 = (dfirst0 + 1) * CH, dnext1 = (dfirst1 + 1) * CH;  // first positions of the next child chunks
   const float pcmin = sel3(cmin[0], cmin[1], cmin[2], axis < 0 ? 0 : axis);
   const float pscl = sel3(scl[0], scl[1], scl[2], axis < 0 ? 0 : axis);
-  // stable partition of the chunk, a stage at a time; the records of children
-  // that are big nodes too are binned for them on the way.  A thread takes up
-  // to 8 consecutive records: runs of one cell (the records of a building, a
-  // wall) mostly lie within a thread or its neighbours, so that one scan of 12
-  // words by shuffles, which bound this step, serves 256 records and not 32.
-  int lrun = 0, rrun = 0;
-  for (int g = 0; kStaged && g * kStage < rn; ++g) {
-    const int m = min(kStage, rn - g * kStage);
+  // stable partition of the chunk; the records of children that are big nodes
+  // too are binned for them on the way.  A thread takes up to 8 consecutive
+  // records: runs of one cell (the records of a building, a wall) mostly lie
+  // within a thread or its neighbours, so that one scan of 12 words by
+  // shuffles, which bound this step, serves 256 records and not 32.
+  if (kStaged) {
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const float4* rec = G.rec;
-    const int c = (m + kBlock - 1) / kBlock, k0 = min(tid * c, m), k1 = min(k0 + c, m);
+    const int c = (rn + kBlock - 1) / kBlock, k0 = min(tid * c, rn), k1 = min(k0 + c, rn);
     unsigned fl = 0;  // bit i: record k0 + i goes left
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
@@ -1130,7 +1120,7 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
         const float* q = reinterpret_cast<const float*>(rec + stage_at(k)) + axis;
         left = bin_of(centre(q[0], q[4]), pcmin, pscl, K) < plane;
       } else {
-        left = r0 + g * kStage + k < nl;
+        left = r0 + k < nl;
       }
       fl |= (unsigned)left << (k - k0);
     }
@@ -1151,7 +1141,7 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
       before += w < warp ? v : 0;
       tl += v;
     }
-    int lp = before, rp = k0 - before;  // positions of the thread's next left and right record in the stage
+    int lp = before, rp = k0 - before;  // positions of the thread's next left and right record in the chunk
     CellRun run;
     run.cell = -1;
     run.n = 0;
@@ -1172,7 +1162,7 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
         const float4 lo = rec[stage_at(kk)], hi = rec[stage_at(kk) + 1];
         const float cx = centre(lo.x, hi.x), cy = centre(lo.y, hi.y), cz = centre(lo.z, hi.z);
         const RecCodes rc = rec_codes(lo, hi, cx, cy, cz);
-        const int jj = left ? (lbase + lrun + pos >= dnext0 ? 1 : 0) : (rbase + rrun + pos >= dnext1 ? 1 : 0);
+        const int jj = left ? (lbase + pos >= dnext0 ? 1 : 0) : (rbase + pos >= dnext1 ? 1 : 0);
         int cell = (left ? 0 : 2) + jj;
         const unsigned cb = (unsigned)cell * kCntStride, bb = left ? 0u : (unsigned)kBinWords;
         unsigned off[3];
@@ -1199,21 +1189,18 @@ __device__ void top_chunk(const BuildArgs& A, TopSmem& S, const TopTask& T, int 
     if (top0 || top1) run_add_warp(run, &S.cbins[0][0], &S.ccnt[0][0][0]);
     __syncthreads();
     // the records leave in the order of their places, 512 bytes a warp
-    for (int i = tid; i < 2 * m; i += kBlock) {
+    for (int i = tid; i < 2 * rn; i += kBlock) {
       const int p = i >> 1;
       const bool left = p < tl;
-      const int dest = left ? lbase + lrun + p : rbase + rrun + p - tl;
+      const int dest = left ? lbase + p : rbase + p - tl;
       const float4 v = rec[stage_at(G.order[p]) + (i & 1)];
       if (dest < (left ? nl : nr))
         dst[2 * ((size_t)T.begin + (left ? 0 : nl) + dest) + (i & 1)] = v;
       else
         set_status(A.ctl, kStBadSplit, 3);
     }
-    lrun += tl;
-    rrun += m - tl;
-    __syncthreads();  // the stage is free
-    fetch(g + 1);
   }
+  int lrun = 0, rrun = 0;
 #pragma unroll
   for (int r = 0; !kStaged && r < kRegRpt; ++r) {  // a round of 256 records, a record a thread
     if (r >= A.rpt || r * kBlock >= rn) break;
