@@ -39,7 +39,6 @@ struct rt_batch_s {
   int* skip[RT_BATCH_MAX_ORDER + 1] = {};
   int* src[RT_BATCH_MAX_ORDER + 1] = {};
   int* counts = nullptr;  // device: rays of order k at counts[k] (k >= 1)
-  int* blocks = nullptr;  // reflect block counts
   rt_ray* seg = nullptr;  // visibility segments, transmitter-major
   uint8_t* occl = nullptr;
   int* flagged = nullptr;  // device: flagged rays of the last walk
@@ -131,7 +130,7 @@ void free_batch(rt_batch_s* b) {
     if (b->skip[k]) cudaFree(b->skip[k]);
     if (b->src[k]) cudaFree(b->src[k]);
   }
-  void* p[] = {b->counts, b->blocks, b->seg, b->occl, b->flagged};
+  void* p[] = {b->counts, b->seg, b->occl, b->flagged};
   for (void* q : p)
     if (q) cudaFree(q);
   drop_graph(b);
@@ -282,7 +281,6 @@ static int rt_batch_create_body(rt_scene scene, const rt_batch_desc* d, rt_batch
       e = cudaMemcpyAsync(b->param_dev, gp.data(), b->n_tx * sizeof(long long), cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);  // off and gp are host temporaries
   }
-  if (e == cudaSuccess) e = alloc(&b->blocks, total / 256 + 2);
   if (e == cudaSuccess) e = alloc(&b->flagged, 1);
   if (e == cudaSuccess && b->n_seg > 0) {
     e = alloc(&b->seg, b->n_seg);
