@@ -4,7 +4,7 @@ Sec. II.C, Fig. 2), scored by the float64 checker.
 The device does not sweep every object split (reading c6).  Its candidate
 set at a node of n records is:
 
-* n > 32 (big-node chunks, CTA splits, warp splits in global memory): for each
+* n > 32 (big-node chunks, CTA splits, single warps in large scenes): for each
   axis, `bins` equal slabs of the node's centroid interval [cmin, cmax]; the
   candidate at plane p (1 <= p < bins) sends left the records whose slab index
   is below p.  Centre = (lo + hi) * 0.5 of the triangle's box, slab index =
