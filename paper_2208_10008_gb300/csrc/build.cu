@@ -637,8 +637,13 @@ __global__ void __launch_bounds__(kBlock) k_prep(BuildArgs A) {
   for (int i = gt; i < n; i += gs) {
     const int t = A.sel ? __ldg(A.sel + i) : i;
     const float4 a = A.tri[3 * (size_t)t], b = A.tri[3 * (size_t)t + 1], c = A.tri[3 * (size_t)t + 2];
-    const float lx = fminf(a.x, fminf(b.x, c.x)), ly = fminf(a.y, fminf(b.y, c.y)), lz = fminf(a.z, fminf(b.z, c.z));
-    const float hx = fmaxf(a.x, fmaxf(b.x, c.x)), hy = fmaxf(a.y, fmaxf(b.y, c.y)), hz = fmaxf(a.z, fmaxf(b.z, c.z));
+    float lx = fminf(a.x, fminf(b.x, c.x)), ly = fminf(a.y, fminf(b.y, c.y)), lz = fminf(a.z, fminf(b.z, c.z));
+    float hx = fmaxf(a.x, fmaxf(b.x, c.x)), hy = fmaxf(a.y, fmaxf(b.y, c.y)), hz = fmaxf(a.z, fmaxf(b.z, c.z));
+    // no ray meets a triangle whose three vertices have no number on an axis;
+    // its box is a point there, or every union with it would be lost
+    if (isnan(lx)) lx = hx = 0.f;
+    if (isnan(ly)) ly = hy = 0.f;
+    if (isnan(lz)) lz = hz = 0.f;
     A.rec[0][2 * (size_t)i] = make_float4(lx, ly, lz, __int_as_float(t));
     A.rec[0][2 * (size_t)i + 1] = make_float4(hx, hy, hz, 0.f);
     const float cx = centre(lx, hx), cy = centre(ly, hy), cz = centre(lz, hz);
