@@ -2456,7 +2456,9 @@ __device__ __forceinline__ bool ref_ok(const BuildArgs& A, int ref, int epoch) {
 // its extent; each lower plane takes the largest byte whose decoded value is
 // not above it, each upper plane the smallest not below it (checked with
 // qplane itself, so the decoded box contains the exact one); when 255 steps
-// fall short after rounding, e grows.
+// fall short after rounding, e grows.  An infinite plane is coded as the
+// largest float's (lower ones) or decodes to infinity (upper ones, at the
+// largest step), beyond every finite ray either way.
 __device__ QNode quantize_node(const WNode& w) {
   const float lo[3][4] = {{w.lox.x, w.lox.y, w.lox.z, w.lox.w}, {w.loy.x, w.loy.y, w.loy.z, w.loy.w},
                           {w.loz.x, w.loz.y, w.loz.z, w.loz.w}};
@@ -2478,9 +2480,12 @@ __device__ QNode quantize_node(const WNode& w) {
       ulo = 0.f;
       uhi = 0.f;
     }
+    ulo = fminf(fmaxf(ulo, -FLT_MAX), FLT_MAX);
     int e = -126;
     const float ext = uhi - ulo;
-    if (ext > 0.f) {
+    if (ext > FLT_MAX) {
+      e = 127;
+    } else if (ext > 0.f) {
       int k;
       frexpf(ext * (1.f / 255.f), &k);  // ext / 255 < 2^k
       e = max(-126, min(127, k));

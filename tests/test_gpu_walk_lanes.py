@@ -62,8 +62,6 @@ def _rays(rng, tris, kind):
 @pytest.mark.parametrize("kind", ["axis", "ratio", "scaled", "far", "open", "nonfinite", "huge", "moved"])
 @pytest.mark.parametrize("width,quant", [(4, 0), (8, 0), (4, 1)])
 def test_lanes_that_part(rb, orc, kind, width, quant):
-    if kind == "nonfinite" and quant:
-        pytest.skip("an infinite box has no byte grid")
     rng = np.random.default_rng(7)
     tris = scenes.tiny_city(seed=3).tris.copy()
     rays = _rays(rng, tris, kind)
