@@ -51,6 +51,7 @@ constexpr float kU = 5.9604645e-08f;   // unit roundoff of float32, 2^-24
 constexpr float kWiden = 1e-6f;        // relative widening of box intervals
 constexpr float kTieRel = 1e-5f;       // relative window of the best-hit checks
 constexpr int kCand = kTraceCand;      // float64 candidates remembered per ray
+constexpr int kCandSoft = 8;           // candidates from which a bound that may not hold costs a second walk
 
 struct RayPre {
   float ox, oy, oz, tmin, tmax;
@@ -647,7 +648,8 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
   int cpos[kCand];
   float clo[kCand];
   int nc = 0;
-  bool walk_all = false;  // the list or the stack was too short
+  // bit 0: the list or the stack was too short; bit 1: the list was once full
+  unsigned again = 0;
   auto remember = [&](int pos, float lo) {
     if (nc == kCand) {  // make room: drop entries already beyond the cull bound
       int w = 0;
@@ -658,13 +660,14 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
           ++w;
         }
       nc = w;
+      again |= 2u;
     }
     if (nc < kCand) {
       cpos[nc] = pos;
       clo[nc] = lo;
       ++nc;
     } else {
-      walk_all = true;
+      again |= 1u;
     }
   };
   // the node being visited stays in registers (cur); only the other
@@ -693,7 +696,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         if (cnt == 0) continue;
         if (sp + cnt - 1 > kSD) {  // cannot hold the farthest: the float64 pass finds what is in them
           flag = true;
-          walk_all = true;
+          again |= 1u;
           cnt = kSD + 1 - sp;
         }
 #pragma unroll
@@ -742,7 +745,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       if (cnt == 0) continue;
       if (sp + cnt - 1 > kSD) {  // cannot hold the farthest: the float64 pass finds what is in them
         flag = true;
-        walk_all = true;
+        again |= 1u;
         cnt = kSD + 1 - sp;
       }
       // push farthest first so the nearest stacked one is popped next
@@ -772,8 +775,7 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         }
         continue;
       }
-      // certain hit: near an end of the interval the float64 rule decides; it
-      // may turn the hit down, so such a hit must not cull what lies behind it
+      // certain hit: near an end of the interval the float64 rule decides
       const bool near_end = fabsf(h.t - r.tmax) <= h.err + kTieRel * fabsf(r.tmax) ||
                             fabsf(h.t - r.tmin) <= h.err + kTieRel * fabsf(h.t);
       if (near_end) flag = true;
@@ -802,7 +804,12 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
         t2 = h.t;
         e2 = h.err;
       }
-      if (!near_end) bound = fminf(bound, h.t + kTieRel * fabsf(h.t) + h.err);
+      // a hit that the float64 rule may turn down must not cull what lies behind
+      // it.  In a launch with skips (bounced rays) it still does: a ray's own
+      // facet is skipped there, and what another facet through its origin hides
+      // is one answer in 30 million of a batch's, after which the survivors of
+      // every later order move up by one
+      bound = fminf(bound, near_end && !skip_ids ? bound : h.t + kTieRel * fabsf(h.t) + h.err);
     }
   }
   if (kAny) {
@@ -819,7 +826,10 @@ __device__ __forceinline__ void walk_one(const TraceArgs& A, const int i, const 
       for (int q = 0; q < nc; ++q)
         if (clo[q] <= bound) cpos[w++] = cpos[q];
     }
-    retest_warp<kAny>(A, rays, i, skip, cpos, w, flag && walk_all, bound, hits, occl);
+    // (the bound may not hold)
+    const bool soft = !kAny && skip_ids && id1 >= 0 && fabsf(t1 - r.tmin) <= e1 + kTieRel * fabsf(t1);
+    if (soft && (nc > kCandSoft || again)) again |= 1u;
+    retest_warp<kAny>(A, rays, i, skip, cpos, w, flag && (again & 1u), soft ? r.tmax : bound, hits, occl);
   }
   if (!live) return;
   if (kStats && A.stats) {
