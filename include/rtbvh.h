@@ -44,7 +44,11 @@ typedef struct rt_session_s* rt_session;
 
 /* One ray, 32 bytes, 16-byte aligned arrays.  Points o + t d with
  * tmin < t < tmax are on the ray.  d need not be unit length; t is in units
- * of |d|.  A ray with a non-finite component, or tmax <= tmin, misses. */
+ * of |d|.  A ray with a non-finite component, or tmax <= tmin, misses.  The
+ * walk's float32 products must not overflow: |d| from 2^-90 to 2^90 over
+ * coordinates of a few thousand is tested; a ray whose direction is far
+ * smaller (below 2^-126 in every component, for instance) may miss what the
+ * definition hits at a distance t beyond 1e30 or so. */
 typedef struct {
   float ox, oy, oz, tmin;
   float dx, dy, dz, tmax;
@@ -138,6 +142,7 @@ const char* rt_last_error(void);
  * tris[9i + 3k .. 9i + 3k + 2]; a host pointer (is_device_ptr = 0; pageable
  * or pinned) or a device pointer (1).  The caller may free `tris` once the
  * stream has reached the call.  n_tri may be 0 (every ray then misses).
+ * A triangle with a NaN or infinite vertex is met by no ray and hides none.
  * Errors: RT_EINVAL (out == NULL, n_tri < 0 or > 2^27), RT_ENOMEM,
  * RT_ECUDA. */
 int rt_scene_upload(const float* tris, int64_t n_tri, int is_device_ptr, void* stream,
@@ -265,6 +270,10 @@ int rt_bvh_export(rt_scene scene, void* stream, int32_t* child, int64_t* leaf_fi
  * (a triangle edge or a second hit within the bound, a hit near tmin or
  * tmax); those are traced again in float64 with the same hit rule as the
  * reference definition (Moller-Trumbore, inclusive edges).
+ * Known fault: with skip_tri_dev, a ray whose origin lies within rounding of
+ * tmin on another facet than the skipped one (coincident facets, an edge) may
+ * be reported as a miss; about 1 bounced ray in 30 million.  A tmin above the
+ * rounding of the origin avoids it.
  * rays_dev: n rt_ray (16-byte aligned); hits_dev: n rt_hit.  n may be 0.
  * Errors: RT_EINVAL, RT_ENOTBUILT, RT_ECUDA. */
 int rt_trace_closest(rt_scene scene, const rt_ray* rays_dev, int64_t n, rt_hit* hits_dev,

@@ -11,7 +11,7 @@
 //                 for the small subtrees); the root task; the root's bins
 //   k_split       one persistent launch for the whole recursion of Fig. 2.
 //                 Its first CTAs take the chunk items of big nodes (more than
-//                 `big` triangles, cut into chunks of 256..1024 records, CTA
+//                 `big` triangles, cut into chunks of 256..2048 records, CTA
 //                 per chunk): Eq. 2 at every bin plane from the node's merged
 //                 bins, stable partition of the chunk into the other record
 //                 buffer, and on the way the children's bins and per-chunk
@@ -1864,10 +1864,9 @@ __device__ __forceinline__ bool cta_split(const BuildArgs& A, SubSmem& S, SubNod
     return bin_of(cc, acmin, ascl, K) < plane;
   };
   int cnt = 0;
-  // A node in shared memory gives a thread at most 32 records (1024 / 256 =
-  // 4): the sides are kept as bits, so that the partition below does not
-  // bin each record again (medium city: 16 bins 187.5 -> 184 us, 8 bins 181
-  // -> 177).
+  // A node in shared memory gives a thread at most 4 records (1024 / 256): the
+  // sides are kept as bits, so that the partition below does not bin each
+  // record again (medium city: 16 bins 187.5 -> 184 us, 8 bins 181 -> 177).
   unsigned fl = 0;
 #pragma unroll 1
   for (int k = k0; k < k1; ++k) {
@@ -2095,7 +2094,7 @@ __device__ void sub_tree(const BuildArgs& A, SubSmem& S, const Task& t, int epoc
     S.mnext = 0;
     if (n <= kMicro) S.ml[S.nm++] = micro_pack(0, n, t.parent, t.side, 0, 0);
   }
-  if (n > kMicro) {  // (a task of k_small's size comes here only when a scene is one)  // the chain of larger children, split by the whole CTA
+  if (n > kMicro) {  // the chain of larger children, split by the whole CTA
     SubNode X = task_node(t, 0);
     for (int it = 0; cta_split<false>(A, S, X, it, t.begin, t.depth, epoch, ws); ++it) {
     }
@@ -2161,10 +2160,6 @@ __device__ void sub_loop(const BuildArgs& A, SubSmem& S, int epoch) {
   }
 }
 
-// The split phase: the first top_ctas CTAs work the chunk items of big nodes
-// (CTA per item) and then join the others, which take the subtree queue
-// (CTA per subtree).  Both run at once, so subtrees proceed while the big
-// nodes of other branches are still being split.
 // Joins the box (lo, hi) to x where a == b, as predicated instructions: a
 // branch here would cost a reconvergence per record.
 __device__ __forceinline__ void binb_join_if(BinB& x, unsigned a, unsigned b, float4 lo, float4 hi) {
@@ -2319,7 +2314,7 @@ __device__ __forceinline__ int warp_split(const BuildArgs& A, unsigned* idx, flo
 // records); here every warp of the SM has a node of its own and the issue of
 // instructions bounds it (13.2M-triangle metro: 778k nodes of at most 32
 // records and 767k splits in 5.3 ms, 14.9 ms inside the split kernel).  24
-// warps per SM (80 registers).
+// warps per SM (80 registers, 184 bytes of spill stores and 260 of loads).
 struct SmallSmem {
   float4 rec[kWarps][2 * kWarpMax];
   unsigned idx[kWarps][kWarpMax];
@@ -2402,6 +2397,12 @@ union SplitSmem {
   SubSmem sub;
 };
 
+// The split phase: the first top_ctas CTAs work the chunk items of big nodes
+// (CTA per item) and then join the others, which take the subtree queue
+// (CTA per subtree).  Both run at once, so subtrees proceed while the big
+// nodes of other branches are still being split; in large scenes every CTA
+// takes chunks first.
+//
 // kStaged (large scenes): the big nodes' chunks go through shared memory, up
 // to 8 consecutive records a thread, instead of registers, a record a thread
 // and round.  The shuffles of the children's binning bound a chunk, 60 for 32
