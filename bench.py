@@ -618,15 +618,15 @@ def run_served(rtbvh, torch, seconds, repeats=3, pool_gib=1.0):
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture of the current kernels (profiles/); None until captured.
 NCU_TRAFFIC_LARGE = {
-    0.7: (278.783061e6 + 174.321749e6, "ncu capture of k_trace<0,0,128,64,0,4> on the 4 x 2^21 metro rays, "
+    0.7: (278.364672e6 + 193.757056e6, "ncu capture of k_trace<0,0,128,64,0,4> on the 4 x 2^21 metro rays, "
                                         "alpha 0.7 tree, mean of 3 launches (profiles/k_trace_metro.md)"),
-    1.0: (273.930752e6 + 135.460011e6, "ncu capture of k_trace<0,0,128,64,0,4> on the 4 x 2^21 metro rays, "
+    1.0: (273.812651e6 + 143.424512e6, "ncu capture of k_trace<0,0,128,64,0,4> on the 4 x 2^21 metro rays, "
                                         "alpha 1 tree, mean of 3 launches (profiles/k_trace_metro.md)")}
 NCU_TRAFFIC = {
-    "k_split": (0.790016e6 + 0.0, "ncu capture of k_split in the timed steps, medium city, leaf 2, 8 bins "
-                                    "(profiles/k_split_medium_city.md)"),
-    "k_trace": (21.552896e6 + 23296.0, "ncu capture of k_trace<0,0,128,64,0,4> in the timed steps, medium "
-                                       "city (profiles/k_trace_medium_city.md)"),
+    "k_split": (0.804864e6 + 256.0, "ncu capture of k_split on the medium city, leaf 2, 16 bins (0.79 MB with the "
+                                    "tuner's other choice, 8 bins; profiles/k_split_medium_city.md)"),
+    "k_trace": (21.533184e6 + 61440.0, "ncu capture of k_trace<0,0,64,16,0,4> (64-ray tile) on the medium city "
+                                       "(21.55 + 0.02 MB with a 128-ray tile; profiles/k_trace_medium_city.md)"),
 }
 
 
