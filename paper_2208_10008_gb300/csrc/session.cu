@@ -87,8 +87,8 @@ class Pool {
 // Copies of finished hits to the callers' buffers, shared out in pieces
 // between the worker thread and a few helpers: one thread copies to fresh
 // memory at about 12 GB/s (its page faults included), and while it copied no
-// request was admitted.  Twelve requests of 64 MB of hits in all take 6.4 ms
-// with one thread, 2.5 ms with eight.  The helpers live as long as the
+// request was admitted.  Twelve requests of 64 MB of hits in all took 6.2 ms
+// with one thread, 2.7 ms with eight.  The helpers live as long as the
 // session, at most kCopyHelpers and half the machine's threads.
 class Copier {
  public:

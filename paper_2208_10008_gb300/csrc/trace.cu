@@ -477,7 +477,7 @@ struct TreeWalk {
 // own widened slab test.  Returns their number; stops when the next leaf might
 // not fit, and sets *more to false at the end of the tree.  (A cull of the
 // triangles by their distance too takes registers from the walk around it:
-// 1,000,003 segments 508 -> 517 us, a launch of 262,143 random rays 238 -> 244.)
+// 1,000,003 segments 578 -> 620 us, a launch of 262,143 random rays 238 -> 244.)
 static_assert(kCand >= kMaxLeaf, "an empty list holds a leaf");
 __device__ __noinline__ int walk_tree(const TraceArgs& A, const float4* r4, const int skip, float bound, TreeWalk* w,
                                       int* cand, bool* more) {
@@ -535,8 +535,9 @@ __device__ __noinline__ int walk_tree(const TraceArgs& A, const float4* r4, cons
 // cand[0 .. nc); nc < 0: its ray is settled); the candidates of all lanes are
 // dealt out to the 32 lanes, so that a warp with two flagged rays of ten
 // candidates each runs the float64 rule once and not ten times: float64 is
-// what the device has least of, a warp's instruction occupies the SM for 16
-// cycles whatever its lanes.  Rays without a complete list (more) then collect
+// what the device has least of: at its nominal rate (about 2 lanes a cycle
+// and SM) a warp's instruction occupies the SM for 16 cycles whatever its
+// lanes.  Rays without a complete list (more) then collect
 // theirs, a list at a time, from the boxes nearer than bound, where the walk
 // has proved a hit, or the float64 best.  Called by whole warps; not inlined,
 // so that the walk's registers are its own.
